@@ -43,8 +43,19 @@ template <typename R> using cplx = typename cplx_t<R>::type;
 template <typename T> __device__ __forceinline__ T cmk(decltype(T::x) x, decltype(T::x) y) {
   T r; r.x = x; r.y = y; return r;
 }
-template <typename T> __device__ __forceinline__ T cadd(T a, T b) { return cmk<T>(a.x + b.x, a.y + b.y); }
-template <typename T> __device__ __forceinline__ T csub(T a, T b) { return cmk<T>(a.x - b.x, a.y - b.y); }
+// Sums and differences of FP32 values as one packed instruction on the (re, im)
+// pair (the same rounding per component; the FP32 lane rate does not change, the
+// issue slots halve). PK = false keeps two scalar additions (a kernel that
+// measures faster with them asks for it). Products stay scalar: w x mixes the two
+// halves, and the packed form needs as many instructions once the swap is counted.
+template <bool PK = true, typename T> __device__ __forceinline__ T cadd(T a, T b) {
+  if constexpr (PK && sizeof(T) == sizeof(float2)) return __fadd2_rn(a, b);
+  else return cmk<T>(a.x + b.x, a.y + b.y);
+}
+template <bool PK = true, typename T> __device__ __forceinline__ T csub(T a, T b) {
+  if constexpr (PK && sizeof(T) == sizeof(float2)) return __fadd2_rn(a, make_float2(-b.x, -b.y));
+  else return cmk<T>(a.x - b.x, a.y - b.y);
+}
 template <typename T> __device__ __forceinline__ T cmul(T a, T b) {
   return cmk<T>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -53,6 +64,11 @@ template <typename T> __device__ __forceinline__ T cmulc(T a, T b) {
   return cmk<T>(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
 }
 template <typename T> __device__ __forceinline__ T cscale(T a, decltype(T::x) s) { return cmk<T>(a.x * s, a.y * s); }
+// a + s t
+template <bool PK = true, typename T> __device__ __forceinline__ T caxpy(T a, decltype(T::x) s, T t) {
+  if constexpr (PK && sizeof(T) == sizeof(float2)) return __ffma2_rn(t, make_float2(s, s), a);
+  else return cmk<T>(a.x + s * t.x, a.y + s * t.y);
+}
 // acc + a b and acc + conj(a) b as four fused multiply-adds (accumulations)
 template <typename T> __device__ __forceinline__ T cfma(T acc, T a, T b) {
   acc.x = fma(a.x, b.x, acc.x);
@@ -114,71 +130,71 @@ template <int N> __host__ __device__ constexpr int first_radix() {
   return (N % 4 == 0 && N != 4) ? 4 : (N % 2 == 0 ? 2 : (N % 3 == 0 ? 3 : (N % 5 == 0 ? 5 : N)));
 }
 
-template <int N, int NTOP, bool INV, typename R>
+template <int N, int NTOP, bool INV, typename R, bool PK = true>
 __device__ __forceinline__ void dft(cplx<R> (&a)[N], const TwTable<R, NTOP>& tw);
 
-template <int NTOP, bool INV, typename R>
+template <int NTOP, bool INV, typename R, bool PK>
 __device__ __forceinline__ void bfly2(cplx<R> (&a)[2]) {
   const cplx<R> t = a[0];
-  a[0] = cadd(t, a[1]);
-  a[1] = csub(t, a[1]);
+  a[0] = cadd<PK>(t, a[1]);
+  a[1] = csub<PK>(t, a[1]);
 }
 
-template <int NTOP, bool INV, typename R>
+template <int NTOP, bool INV, typename R, bool PK>
 __device__ __forceinline__ void bfly4(cplx<R> (&a)[4]) {
-  const cplx<R> s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]);
-  const cplx<R> s13 = cadd(a[1], a[3]), d13 = rot_q<INV>(csub(a[1], a[3]));
-  a[0] = cadd(s02, s13);
-  a[2] = csub(s02, s13);
-  a[1] = cadd(d02, d13);
-  a[3] = csub(d02, d13);
+  const cplx<R> s02 = cadd<PK>(a[0], a[2]), d02 = csub<PK>(a[0], a[2]);
+  const cplx<R> s13 = cadd<PK>(a[1], a[3]), d13 = rot_q<INV>(csub<PK>(a[1], a[3]));
+  a[0] = cadd<PK>(s02, s13);
+  a[2] = csub<PK>(s02, s13);
+  a[1] = cadd<PK>(d02, d13);
+  a[3] = csub<PK>(d02, d13);
 }
 
 // radix 3: X1,2 = a0 + c (a1 + a2) -/+ i s (a1 - a2) with w_3 = c - i s (forward)
-template <int NTOP, bool INV, typename R>
+template <int NTOP, bool INV, typename R, bool PK>
 __device__ __forceinline__ void bfly3(cplx<R> (&a)[3], const TwTable<R, NTOP>& tw) {
   const cplx<R> w3 = tw.w[NTOP / 3];
   const R c = w3.x, s = -w3.y;
-  const cplx<R> t = cadd(a[1], a[2]);
-  const cplx<R> d = cscale(csub(a[1], a[2]), s);
-  const cplx<R> u = cmk<cplx<R>>(a[0].x + c * t.x, a[0].y + c * t.y);
-  a[0] = cadd(a[0], t);
+  const cplx<R> t = cadd<PK>(a[1], a[2]);
+  const cplx<R> d = cscale(csub<PK>(a[1], a[2]), s);
+  const cplx<R> u = caxpy<PK>(a[0], c, t);
+  a[0] = cadd<PK>(a[0], t);
   const cplx<R> rd = rot_q<INV>(d);
-  a[1] = cadd(u, rd);
-  a[2] = csub(u, rd);
+  a[1] = cadd<false>(u, rd);   // scalar: s (a1 - a2) and the sum are one FMA each
+  a[2] = csub<false>(u, rd);
 }
 
 // radix 5 with c1 = cos 2pi/5, c2 = cos 4pi/5, s1 = sin 2pi/5, s2 = sin 4pi/5
-template <int NTOP, bool INV, typename R>
+template <int NTOP, bool INV, typename R, bool PK>
 __device__ __forceinline__ void bfly5(cplx<R> (&a)[5], const TwTable<R, NTOP>& tw) {
   const cplx<R> w1 = tw.w[NTOP / 5], w2 = tw.w[2 * NTOP / 5];
   const R c1 = w1.x, s1 = -w1.y, c2 = w2.x, s2 = -w2.y;
-  const cplx<R> t1 = cadd(a[1], a[4]), t2 = cadd(a[2], a[3]);
-  const cplx<R> t3 = csub(a[1], a[4]), t4 = csub(a[2], a[3]);
+  const cplx<R> t1 = cadd<PK>(a[1], a[4]), t2 = cadd<PK>(a[2], a[3]);
+  const cplx<R> t3 = csub<PK>(a[1], a[4]), t4 = csub<PK>(a[2], a[3]);
   const cplx<R> b1 = cmk<cplx<R>>(a[0].x + c1 * t1.x + c2 * t2.x, a[0].y + c1 * t1.y + c2 * t2.y);
   const cplx<R> b2 = cmk<cplx<R>>(a[0].x + c2 * t1.x + c1 * t2.x, a[0].y + c2 * t1.y + c1 * t2.y);
   const cplx<R> e1 = rot_q<INV>(cmk<cplx<R>>(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y));
   const cplx<R> e2 = rot_q<INV>(cmk<cplx<R>>(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y));
-  a[0] = cadd(a[0], cadd(t1, t2));
-  a[1] = cadd(b1, e1);
-  a[4] = csub(b1, e1);
-  a[2] = cadd(b2, e2);
-  a[3] = csub(b2, e2);
+  a[0] = cadd<PK>(a[0], cadd<PK>(t1, t2));
+  a[1] = cadd<PK>(b1, e1);
+  a[4] = csub<PK>(b1, e1);
+  a[2] = cadd<PK>(b2, e2);
+  a[3] = csub<PK>(b2, e2);
 }
 
-template <int N, int NTOP, bool INV, typename R>
+template <int N, int NTOP, bool INV, typename R, bool PK>
 __device__ __forceinline__ void dft(cplx<R> (&a)[N], const TwTable<R, NTOP>& tw) {
   static_assert(NTOP % N == 0, "sub-length must divide the table length");
   if constexpr (N == 1) {
     return;
   } else if constexpr (N == 2) {
-    bfly2<NTOP, INV, R>(a);
+    bfly2<NTOP, INV, R, PK>(a);
   } else if constexpr (N == 3) {
-    bfly3<NTOP, INV, R>(a, tw);
+    bfly3<NTOP, INV, R, PK>(a, tw);
   } else if constexpr (N == 4) {
-    bfly4<NTOP, INV, R>(a);
+    bfly4<NTOP, INV, R, PK>(a);
   } else if constexpr (N == 5) {
-    bfly5<NTOP, INV, R>(a, tw);
+    bfly5<NTOP, INV, R, PK>(a, tw);
   } else {
     constexpr int RX = first_radix<N>();
     static_assert(RX != N, "unsupported prime factor");
@@ -189,16 +205,38 @@ __device__ __forceinline__ void dft(cplx<R> (&a)[N], const TwTable<R, NTOP>& tw)
 #pragma unroll
       for (int m = 0; m < M; ++m) sub[r][m] = a[r + RX * m];
 #pragma unroll
-    for (int r = 0; r < RX; ++r) dft<M, NTOP, INV, R>(sub[r], tw);
+    for (int r = 0; r < RX; ++r) dft<M, NTOP, INV, R, PK>(sub[r], tw);
 #pragma unroll
     for (int k = 0; k < M; ++k) {
       cplx<R> t[RX];
 #pragma unroll
       for (int r = 0; r < RX; ++r) t[r] = twiddle<N, NTOP, INV, R>(sub[r][k], r * k, tw);
-      dft<RX, NTOP, INV, R>(t, tw);
+      dft<RX, NTOP, INV, R, PK>(t, tw);
 #pragma unroll
       for (int q = 0; q < RX; ++q) a[k + M * q] = t[q];
     }
+  }
+}
+
+// A whole line in one thread by a radix-2 step over the even and odd samples:
+// the operations of the two-lane form (split_line_dft), in the same order, so
+// the two give the same bits.
+template <int N, bool INV, typename R>
+__device__ __forceinline__ void line_dft2(cplx<R> (&a)[N], const TwTable<R, N>& tw) {
+  constexpr int M = N / 2;
+  cplx<R> e[M], o[M];
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    e[m] = a[2 * m];
+    o[m] = a[2 * m + 1];
+  }
+  dft<M, N, INV, R>(e, tw);
+  dft<M, N, INV, R>(o, tw);
+#pragma unroll
+  for (int k = 0; k < M; ++k) {
+    const cplx<R> t = k == 0 ? o[k] : 4 * k == N ? rot_q<INV>(o[k]) : cmul(o[k], twiddle_value<N, N, INV, R>(k, tw));
+    a[k] = cadd(e[k], t);
+    a[k + M] = csub(e[k], t);
   }
 }
 

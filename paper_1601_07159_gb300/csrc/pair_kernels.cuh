@@ -28,7 +28,7 @@
 // are compiled in. On cubic grids passes B and D use instances with the grid
 // compiled in (strides and offsets folded into the instructions). At the
 // larger edges a line is held by two lanes instead of one thread
-// (split_line_dft): the plane passes when the longer plane edge is >= 48
+// (split_line_dft): the plane passes when the longer plane edge is >= 96
 // (FP64: >= 64), FP64 pass B from n_z = 64; FP32 pencils of 64 and 96 are
 // spread over four warps (pass_b_quad_kernel).
 //
@@ -242,13 +242,33 @@ template <typename R, int NZ, bool CUBE> struct PencilGeom {
 
 template <int NX, int NY> constexpr int kMaxLine = NX > NY ? NX : NY;
 
+// Items (pair, z-plane) per CTA of the whole-line plane kernels. FP32: about 128
+// threads (two planes of 48 or 64, five of 24), so that several independent
+// blocks share an SM and one block's loads run under another's transforms;
+// about 256 threads left one or two blocks per SM that loaded, transformed and
+// stored together (a 64-pair tile, passes A + C: 24^3 8.3 -> 7.3, 32^3 6.0 ->
+// 5.0, 36^3 7.3 -> 6.6 ps per pair point). FP64: about 256 threads, <= 96 KB.
 template <typename R, int NX, int NY> __host__ __device__ constexpr int plane_items() {
-  // items (pair, z-plane) per CTA of the plane kernels: ~256 threads, <= 96 KB
   constexpr int ML = kMaxLine<NX, NY>;
-  constexpr int by_threads = (256 / ML) > 0 ? (256 / ML) : 1;
+  constexpr int want = sizeof(R) == 4 ? 128 : 256;
+  constexpr int by_threads = (want / ML) > 0 ? (want / ML) : 1;
   constexpr int by_smem = (96 * 1024) / (NY * (NX + 1) * (int)sizeof(cplx<R>));
   constexpr int v = by_threads < by_smem ? by_threads : by_smem;
   return v > 0 ? v : 1;
+}
+// Whole-line planes that transform their lines radix 2 first: FP32 planes whose
+// longer edge is at least 48 (results equal to the bit to the two-lane form).
+template <typename R, int NX, int NY> constexpr bool kLine2 =
+    sizeof(R) == 4 && kMaxLine<NX, NY> >= 48 && NX % 4 == 0 && NY % 4 == 0;
+
+// Blocks per SM those kernels are compiled for: FP32 lines need about 2 ML + 28
+// registers (the line itself and the butterflies' temporaries), and more blocks
+// would spill; FP64 two.
+template <typename R, int NX, int NY> __host__ __device__ constexpr int plane_blocks() {
+  constexpr int ML = kMaxLine<NX, NY>;
+  constexpr int warps = (ML * plane_items<R, NX, NY>() + 31) / 32;
+  constexpr int v = 65536 / (32 * warps * (2 * ML + 28));
+  return sizeof(R) == 4 ? (v < 1 ? 1 : v > 8 ? 8 : v) : 2;
 }
 constexpr int kEngineThreads = 256;
 template <typename R, int N> __host__ __device__ constexpr int engine_items() {
@@ -260,8 +280,14 @@ template <typename R, int N> __host__ __device__ constexpr int engine_items() {
 }
 
 // ---------------------------------------------------------------- pass bodies
+// A whole line in registers: radix 2 first (LINE2) or by the radix order.
+template <int N, bool INV, bool LINE2, typename R>
+__device__ __forceinline__ void line_dft(cplx<R> (&a)[N], const TwTable<R, N>& tw) {
+  if constexpr (LINE2) line_dft2<N, INV, R>(a, tw);
+  else dft<N, N, INV, R>(a, tw);
+}
 // Pass A on virtual block `vb` (IPB plane items, thread tid = ty * max(NX, NY) + tx).
-template <typename R, int NX, int NY, bool REAL, bool COH, int IPB, bool PDL>
+template <typename R, int NX, int NY, bool REAL, bool COH, int IPB, bool PDL, bool LINE2>
 __device__ __forceinline__ void body_a(const PlaneParams<R, NX, NY>& P, const TileDesc* tiles, int ntiles,
                                        int npairs, cplx<R>* smem, long long vb, int tid) {
   constexpr int ML = kMaxLine<NX, NY>;
@@ -298,7 +324,7 @@ __device__ __forceinline__ void body_a(const PlaneParams<R, NX, NY>& P, const Ti
         a[y] = cmulc(xv, yv);                 // conj(x_l) * y_r
       }
     }
-    dft<NY, NY, false, R>(a, P.tw.ty());      // along y, column x = tx
+    line_dft<NY, false, LINE2, R>(a, P.tw.ty());   // along y, column x = tx
 #pragma unroll
     for (int k = 0; k < NY; ++k) buf[k * (NX + 1) + tx] = a[k];
   }
@@ -307,7 +333,7 @@ __device__ __forceinline__ void body_a(const PlaneParams<R, NX, NY>& P, const Ti
     cplx<R> b[NX];
 #pragma unroll
     for (int x = 0; x < NX; ++x) b[x] = buf[tx * (NX + 1) + x];
-    dft<NX, NX, false, R>(b, P.tw.tx());      // along x, row ky = tx
+    line_dft<NX, false, LINE2, R>(b, P.tw.tx());   // along x, row ky = tx
     if constexpr (PDL) griddep_wait();        // the previous batch's pass D still reads S
     cplx<R>* out = P.S + ((long long)p * P.nz + z) * NX * NY + tx;
 #pragma unroll
@@ -363,7 +389,7 @@ __device__ __forceinline__ void body_b(const PencilParams<R, NZ>& P, const TileD
 }
 
 // Pass C on virtual block `vb` (IPB plane items).
-template <typename R, int NX, int NY, bool COH, int IPB>
+template <typename R, int NX, int NY, bool COH, int IPB, bool LINE2>
 __device__ __forceinline__ void body_c(const PlaneParams<R, NX, NY>& P, int npairs, cplx<R>* smem, long long vb,
                                        int tid) {
   constexpr int ML = kMaxLine<NX, NY>;
@@ -381,7 +407,7 @@ __device__ __forceinline__ void body_c(const PlaneParams<R, NX, NY>& P, int npai
     cplx<R> b[NX];
 #pragma unroll
     for (int kx = 0; kx < NX; ++kx) b[kx] = ldx<COH>(plane + kx * NY + tx);   // row ky = tx
-    dft<NX, NX, true, R>(b, P.tw.tx());                                      // inverse along x
+    line_dft<NX, true, LINE2, R>(b, P.tw.tx());                              // inverse along x
 #pragma unroll
     for (int x = 0; x < NX; ++x) buf[tx * (NX + 1) + x] = b[x];
   }
@@ -390,7 +416,7 @@ __device__ __forceinline__ void body_c(const PlaneParams<R, NX, NY>& P, int npai
     cplx<R> a[NY];
 #pragma unroll
     for (int ky = 0; ky < NY; ++ky) a[ky] = buf[ky * (NX + 1) + tx];  // column x = tx
-    dft<NY, NY, true, R>(a, P.tw.ty());                               // inverse along y
+    line_dft<NY, true, LINE2, R>(a, P.tw.ty());                       // inverse along y
 #pragma unroll
     for (int y = 0; y < NY; ++y) stx<COH>(plane + y * NX + tx, a[y]);
   }
@@ -799,11 +825,11 @@ __device__ __forceinline__ void body_d(const PointParams<R>& P, const TileDesc& 
 
 // ---------------------------------------------------------------- four-kernel mode
 template <typename R, int NX, int NY, bool REAL>
-__global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), 2)
+__global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), plane_blocks<R, NX, NY>())
 pass_a_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   griddep_launch();
-  body_a<R, NX, NY, REAL, false, plane_items<R, NX, NY>(), true>(
+  body_a<R, NX, NY, REAL, false, plane_items<R, NX, NY>(), true, kLine2<R, NX, NY>>(
       P, P.tiles, P.ntiles, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x, threadIdx.x);
 }
 
@@ -841,14 +867,14 @@ __device__ __forceinline__ void split_combine(const cplx<R> (&a)[N / 2], int h, 
     const C od = h ? a[H + j] : recv;                    // O[hH + j]
     const C w = csel<R>(h, twiddle_value<N, N, INV, R>(H + j, tw), twiddle_value<N, N, INV, R>(j, tw));
     const C t = cmul(od, w);
-    sink(j, cadd(ev, t));
-    sink(H + j, csub(ev, t));
+    sink(j, cadd<false>(ev, t));
+    sink(H + j, csub<false>(ev, t));
   }
 }
 template <int N, bool INV, typename R>
 __device__ __forceinline__ void split_line_dft(cplx<R> (&a)[N / 2], cplx<R> (&y)[N / 2], int h,
                                                const TwTable<R, N>& tw) {
-  dft<N / 2, N, INV, R>(a, tw);                            // E (lane 0) or O (lane 1)
+  dft<N / 2, N, INV, R, false>(a, tw);                     // E (lane 0) or O (lane 1)
   split_combine<N, INV, R>(a, h, tw, [&](int j, cplx<R> v) { y[j] = v; });
 }
 // Pass B for the large FP64 pencils (n_z >= 64), whose whole pencil per thread
@@ -938,24 +964,21 @@ pass_b_split_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
   }
 }
 
-// Planes whose passes use the two-lane line transforms (one plane per block),
-// and the blocks per SM their launch bounds ask for: at 48^3 the half-length
-// lines need 72-95 registers, so six 96-thread blocks (18-27 warps) fit an SM
-// where the one-thread-per-line form runs 15 warps at 117-128. Below 48 the
-// whole-line form is as fast (several planes per block). Pass A at 48^3 is held
-// to 80 registers (eight blocks, 24 warps): 1.3 % faster steps. FP64 lines take
-// the two-lane form from 64 (a whole FP64 line of 64 would not fit a thread's
-// registers), with one or two blocks per SM.
-constexpr int kSplitMinEdge = 48;
+// Planes whose passes use the two-lane line transforms (one plane per block):
+// the lines that do not fit a thread's registers beside enough warps. A whole
+// FP32 line of 64 needs 168 registers (three 128-thread blocks, 12 warps per
+// SM) and still beats the two-lane form, whose selects and shuffles are 40 % of
+// its instructions: 64^3 A 60.4 -> 51.8, C 59.4 -> 55.3 us per 64-pair tile,
+// 48^3 25.6 -> 21.3 and 20.5 -> 18.4. At 96 (234 registers, six warps) it
+// loses: A 207 -> 223, C 188 -> 213. FP64 lines take the two-lane form from 64,
+// with one or two blocks per SM.
+constexpr int kSplitMinEdge = 96;
 constexpr int kSplitMinEdgeF64 = 64;
 template <typename R, int NX, int NY> constexpr bool kSplitPlanes =
     NX % 4 == 0 && NY % 4 == 0 &&
     (sizeof(R) == 4 ? kMaxLine<NX, NY> >= kSplitMinEdge : kMaxLine<NX, NY> >= kSplitMinEdgeF64);
 template <typename R, int NX, int NY> constexpr int kSplitBlocks =
-    sizeof(R) == 8 ? (kMaxLine<NX, NY> >= 96 ? 1 : 2)
-                   : (kMaxLine<NX, NY> >= 96 ? 2 : kMaxLine<NX, NY> >= 64 ? 4 : 6);
-template <typename R, int NX, int NY> constexpr int kSplitBlocksA =
-    sizeof(R) == 4 && NX == 48 && NY == 48 ? 8 : kSplitBlocks<R, NX, NY>;
+    sizeof(R) == 8 && kMaxLine<NX, NY> >= 96 ? 1 : 2;
 template <typename R, int NX, int NY> constexpr size_t kSplitSmem = (size_t)NY * (NX + 1) * sizeof(cplx<R>);
 
 // frequency index held in y[j] by lane h
@@ -969,9 +992,11 @@ template <int N> __device__ __forceinline__ int split_index(int j, int h) {
 // of a whole line per thread (which at 96^3 would need over 200), so more
 // warps per SM hide the latency of the plane loads and stores. On a
 // non-square plane the lanes past the shorter edge compute on zeros and store
-// nothing, so every lane of a warp takes part in the shuffles.
+// nothing, so every lane of a warp takes part in the shuffles. Scalar additions:
+// with packed ones the 96-point passes measured 212 -> 207 (A) but 188 -> 207 us
+// (C) per 64-pair tile.
 template <typename R, int NX, int NY, bool REAL>
-__global__ void __launch_bounds__(2 * kMaxLine<NX, NY>, kSplitBlocksA<R, NX, NY>)
+__global__ void __launch_bounds__(2 * kMaxLine<NX, NY>, kSplitBlocks<R, NX, NY>)
 pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   using C = cplx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1008,7 +1033,7 @@ pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
         a[m] = act ? cmulc(load_vec<R, REAL>(P.X, xo + yy * NX), load_vec<R, REAL>(P.Y, yo + yy * NX)) : zero;
       }
     }
-    dft<M, NY, false, R>(a, P.tw.ty());                   // along y
+    dft<M, NY, false, R, false>(a, P.tw.ty());            // along y
     split_combine<NY, false, R>(a, h, P.tw.ty(), [&](int j, C v) {
       if (act) buf[split_index<NY>(j, h) * (NX + 1) + q] = v;
     });
@@ -1020,7 +1045,7 @@ pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
     C a[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) a[m] = act ? buf[q * (NX + 1) + 2 * m + h] : zero;
-    dft<M, NX, false, R>(a, P.tw.tx());                   // along x
+    dft<M, NX, false, R, false>(a, P.tw.tx());            // along x
     griddep_wait();                                        // the previous batch's pass D still reads S
     C* out = P.S + ((long long)p * P.nz + z) * NX * NY + q;
     split_combine<NX, false, R>(a, h, P.tw.tx(), [&](int j, C v) {
@@ -1048,7 +1073,7 @@ pass_c_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
     C a[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) a[m] = act ? plane[(long long)(2 * m + h) * NY + q] : zero;
-    dft<M, NX, true, R>(a, P.tw.tx());
+    dft<M, NX, true, R, false>(a, P.tw.tx());
     split_combine<NX, true, R>(a, h, P.tw.tx(), [&](int j, C v) {
       if (act) buf[q * (NX + 1) + split_index<NX>(j, h)] = v;   // row ky, column x
     });
@@ -1060,7 +1085,7 @@ pass_c_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
     C a[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) a[m] = act ? buf[(2 * m + h) * (NX + 1) + q] : zero;
-    dft<M, NY, true, R>(a, P.tw.ty());
+    dft<M, NY, true, R, false>(a, P.tw.ty());
     split_combine<NY, true, R>(a, h, P.tw.ty(), [&](int j, C v) {
       if (act) plane[(long long)split_index<NY>(j, h) * NX + q] = v;
     });
@@ -1227,12 +1252,12 @@ pass_b_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
 }
 
 template <typename R, int NX, int NY>
-__global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), 2)
+__global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), plane_blocks<R, NX, NY>())
 pass_c_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   griddep_launch();
   griddep_wait();
-  body_c<R, NX, NY, false, plane_items<R, NX, NY>()>(P, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x,
+  body_c<R, NX, NY, false, plane_items<R, NX, NY>(), kLine2<R, NX, NY>>(P, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x,
                                                      threadIdx.x);
 }
 
@@ -1356,12 +1381,12 @@ pair_engine_kernel(const __grid_constant__ EngineParams<R, N> E) {
     const EngineBatch& b = E.batches[k];
     const TileDesc* tiles = E.pl.tiles + b.toff;
     if (pass == 0) {
-      body_a<R, N, N, REAL, true, IPB, false>(E.pl, tiles, b.ntiles, b.npairs, smem, loc, tid);
+      body_a<R, N, N, REAL, true, IPB, false, false>(E.pl, tiles, b.ntiles, b.npairs, smem, loc, tid);
     } else if (pass == 1) {
       body_b<R, N, true, true>(E.pe, tiles, b.ntiles, b.npairs, E.mode, loc, tid, kEngineThreads, red,
                                E.mode != 0 ? E.pe.Epart + loc : nullptr);
     } else if (pass == 2) {
-      body_c<R, N, N, true, IPB>(E.pl, b.npairs, smem, loc, tid);
+      body_c<R, N, N, true, IPB, false>(E.pl, b.npairs, smem, loc, tid);
     } else {
       const long long nvb = ((long long)N * N * N + kEngineThreads - 1) / kEngineThreads;
       const TileDesc d = tiles[loc / nvb];
