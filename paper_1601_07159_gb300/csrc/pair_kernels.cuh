@@ -833,14 +833,23 @@ pass_a_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
       P, P.tiles, P.ntiles, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x, threadIdx.x);
 }
 
+// The two lanes of a line sit 16 apart: lanes 0-15 of a warp hold the even
+// samples of 16 consecutive lines, lanes 16-31 the odd ones. A half-warp then
+// touches 16 consecutive columns of one row (or one column of 16 consecutive
+// padded rows), which are free of bank conflicts in the plane buffer and whole
+// 128-byte lines in global memory; with neighbouring lanes sharing a line every
+// access of the buffer was a two-way conflict (96^3, one 64-pair tile: A 220 ->
+// 212, C 192 -> 188 us).
+__device__ __forceinline__ int split_line(int tid) { return ((tid >> 5) << 4) | (tid & 15); }
+__device__ __forceinline__ int split_half(int tid) { return (tid >> 4) & 1; }
 template <typename T> __device__ __forceinline__ T shfl_pair(T v) {
   T r;
-  r.x = __shfl_xor_sync(0xffffffffu, v.x, 1);
-  r.y = __shfl_xor_sync(0xffffffffu, v.y, 1);
+  r.x = __shfl_xor_sync(0xffffffffu, v.x, 16);
+  r.y = __shfl_xor_sync(0xffffffffu, v.y, 16);
   return r;
 }
 
-// A length-N transform of a line held by two lanes (lanes 2q, 2q+1): lane h
+// A length-N transform of a line held by two lanes (split_line): lane h
 // holds the samples 2m + h in a[], and on return holds y[j] = Y[hN/4 + j] and
 // y[N/4 + j] = Y[hN/4 + j + N/2] (the forward or inverse DFT, unnormalised):
 // a DFT of N/2 per lane, the lane-1 twiddles w^{+-k}, one shuffle per value
@@ -879,7 +888,7 @@ __device__ __forceinline__ void split_line_dft(cplx<R> (&a)[N / 2], cplx<R> (&y)
 }
 // Pass B for the large FP64 pencils (n_z >= 64), whose whole pencil per thread
 // spills (FP32 pencils of 64 and 96 take the four-warp form, pass_b_quad_kernel):
-// two lanes per z-pencil (lanes 2q, 2q+1 of a warp; 128 pencils per block). Lane h holds the samples z = 2m + h and transforms them with a DFT of
+// two lanes per z-pencil (split_line; 128 pencils per block). Lane h holds the samples z = 2m + h and transforms them with a DFT of
 // N/2:
 //   forward  Y[k] = E[k] + w^k O[k], Y[k + N/2] = E[k] - w^k O[k]
 //            (E, O the half-length transforms of the even / odd samples,
@@ -912,8 +921,8 @@ pass_b_split_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
   griddep_wait();
   const PencilGeom<R, NZ, CUBE> G(P);
   const int nxy = G.nxy;
-  const int tid = threadIdx.x, h = tid & 1;
-  const long long gid = (long long)blockIdx.x * kBSplitPencils + (tid >> 1);
+  const int tid = threadIdx.x, h = split_half(tid);
+  const long long gid = (long long)blockIdx.x * kBSplitPencils + split_line(tid);
   const bool active = gid < (long long)P.npairs * nxy;    // same for both lanes of a pencil
   const int p = active ? (int)(gid / nxy) : 0;
   const int f = active ? (int)(gid % nxy) : 0;
@@ -979,6 +988,7 @@ template <typename R, int NX, int NY> constexpr bool kSplitPlanes =
     (sizeof(R) == 4 ? kMaxLine<NX, NY> >= kSplitMinEdge : kMaxLine<NX, NY> >= kSplitMinEdgeF64);
 template <typename R, int NX, int NY> constexpr int kSplitBlocks =
     sizeof(R) == 8 && kMaxLine<NX, NY> >= 96 ? 1 : 2;
+template <int NX, int NY> constexpr bool kSplitWarps = (2 * kMaxLine<NX, NY>) % 32 == 0;   // whole warps of line pairs
 template <typename R, int NX, int NY> constexpr size_t kSplitSmem = (size_t)NY * (NX + 1) * sizeof(cplx<R>);
 
 // frequency index held in y[j] by lane h
@@ -999,10 +1009,11 @@ template <typename R, int NX, int NY, bool REAL>
 __global__ void __launch_bounds__(2 * kMaxLine<NX, NY>, kSplitBlocks<R, NX, NY>)
 pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   using C = cplx<R>;
+  static_assert(kSplitWarps<NX, NY>, "a line's lanes share a warp");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   griddep_launch();
-  const int tid = threadIdx.x, q = tid >> 1, h = tid & 1;
+  const int tid = threadIdx.x, q = split_line(tid), h = split_half(tid);
   const long long item = blockIdx.x;                      // one (pair, z) plane per block, z-major:
   const int z = (int)(item / P.npairs), p = (int)(item % P.npairs);   // pairs sharing a plane run together
   int l, r, r2 = -1;
@@ -1058,11 +1069,12 @@ template <typename R, int NX, int NY>
 __global__ void __launch_bounds__(2 * kMaxLine<NX, NY>, kSplitBlocks<R, NX, NY>)
 pass_c_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   using C = cplx<R>;
+  static_assert(kSplitWarps<NX, NY>, "a line's lanes share a warp");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   griddep_launch();
   griddep_wait();
-  const int tid = threadIdx.x, q = tid >> 1, h = tid & 1;
+  const int tid = threadIdx.x, q = split_line(tid), h = split_half(tid);
   const long long item = blockIdx.x;
   const int p = (int)(item / P.nz), z = (int)(item % P.nz);
   C* plane = P.S + ((long long)p * P.nz + z) * NX * NY;
