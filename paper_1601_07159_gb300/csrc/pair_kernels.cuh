@@ -21,7 +21,7 @@
 //                           Out_l -= y_r conj(v); registers hold the tile's
 //                           orbitals and accumulators, one read-modify-write of
 //                           each output per tile, fixed summation order (full
-//                           off-diagonal tiles: two threads per point).
+//                           off-diagonal tiles: four threads per point, FP64 two).
 // The plane passes are compiled per (n_x, n_y), the pencil pass per n_z (the
 // pencil's (kx, ky) position is a run-time index), the accumulate pass once per
 // precision; a grid n_x x n_y x n_z runs when its plane and its pencil length
@@ -52,7 +52,7 @@
 // Tiles within a batch touch disjoint outputs (the schedule guarantees it) and
 // batches run in order, so the accumulation needs no atomics and the result is
 // bitwise reproducible. The engine sums a full off-diagonal tile's left
-// outputs in one thread rather than two, so the two modes agree to rounding.
+// outputs in one thread, so the two modes agree to rounding.
 #pragma once
 #include "ace_internal.h"
 #include "fft_reg.cuh"
@@ -544,6 +544,136 @@ __device__ __forceinline__ void d_split_off(const PointParams<R>& P, const TileD
     rmw_out<R, REAL, false>(P.OutX, (long long)(d.l0 + h * H + o) * P.ld + g, cadd(lo, hi), P.scale);
     rmw_out<R, REAL, false>(P.OutY, (long long)(d.r0 + h * H + o) * P.ld + g, ar[o], P.scale);
   }
+}
+
+// Off-diagonal full FP32 tile with four threads per grid point: thread (lh, rh)
+// takes the left orbitals l0 + 4 lh .. + 3 and the right ones r0 + 4 rh .. + 3 (16
+// of the tile's 64 pair potentials), so a thread has half the loads of d_split_off
+// in flight at once and a tile has twice the threads: 64 potentials per thread
+// pair left the launch of a 48^3 tile at 1.4 waves of blocks. The sums are those
+// of d_split_off, in its order, to the bit: the right outputs' sums run over the
+// left orbitals in turn, so the threads lh = 1 continue from the partial sums that
+// lh = 0 leaves in shared memory (their potentials are in registers by then), and
+// the left outputs add the two right halves' sums. Threads lh = 0 then update
+// Out_l (4 rh .. 4 rh + 3), threads lh = 1 Out_r.
+constexpr int kDQuadPts = 64;    // points per 256-thread block
+template <typename R, long long NGC>
+__device__ __forceinline__ void d_quad_off(const PointParams<R>& P, const TileDesc& d, long long vbx, int tid,
+                                           cplx<R>* xch) {
+  using C = cplx<R>;
+  const long long NG = NGC ? NGC : P.ng;
+  constexpr int B = kTileMax, H = kTileMax / 2;
+  const int w = tid >> 5, rh = w & 1, lh = (w >> 1) & 1, pt = ((w >> 2) << 5) | (tid & 31);
+  const long long g = vbx * kDQuadPts + pt;
+  const bool act = g < NG;
+  const C zero = cmk<C>(R(0), R(0));
+  const C* V = P.S + (long long)(d.slot0 + lh * H * B + rh * H) * NG + g;
+  const C* X = static_cast<const C*>(P.X) + (long long)(d.l0 + lh * H) * P.ld + g;
+  const C* Y = static_cast<const C*>(P.Y) + (long long)(d.r0 + rh * H) * P.ld + g;
+  // the output orbitals of this thread: Out_l for lh = 0, Out_r for lh = 1
+  C* O = (lh ? static_cast<C*>(P.OutY) + (long long)d.r0 * P.ld : static_cast<C*>(P.OutX) + (long long)d.l0 * P.ld) +
+         (long long)rh * H * P.ld + g;
+  C v[H][H], xl[H], al[H], ar[H], out[H];
+#pragma unroll
+  for (int li = 0; li < H; ++li)
+#pragma unroll
+    for (int ri = 0; ri < H; ++ri) v[li][ri] = act ? __ldcs(V + (long long)(li * B + ri) * NG) : zero;
+#pragma unroll
+  for (int o = 0; o < H; ++o) {
+    xl[o] = act ? X[(long long)o * P.ld] : zero;
+    al[o] = zero;
+    ar[o] = zero;
+  }
+#pragma unroll
+  for (int ri = 0; ri < H; ++ri) {
+    const C yr = act ? Y[(long long)ri * P.ld] : zero;
+#pragma unroll
+    for (int li = 0; li < H; ++li) al[li] = cfmac(al[li], v[li][ri], yr);
+  }
+#pragma unroll
+  for (int o = 0; o < H; ++o) out[o] = act ? O[(long long)o * P.ld] : zero;
+  // exchange, per point: [0, 4) the right sums so far of rh = 0, [4, 8) of rh = 1,
+  // [8, 12) the left sums of (0, 1), [12, 16) of (1, 0), [16, 20) of (1, 1)
+  C* xp = xch + pt;
+  if (lh == 0) {
+#pragma unroll
+    for (int li = 0; li < H; ++li)
+#pragma unroll
+      for (int ri = 0; ri < H; ++ri) ar[ri] = cfma(ar[ri], xl[li], v[li][ri]);
+#pragma unroll
+    for (int o = 0; o < H; ++o) xp[(rh * H + o) * kDQuadPts] = ar[o];
+  }
+  if (lh | rh) {
+#pragma unroll
+    for (int o = 0; o < H; ++o) xp[((1 + 2 * lh + rh) * H + o) * kDQuadPts] = al[o];
+  }
+  __syncthreads();
+  if (!act) return;
+  if (lh == 0) {
+#pragma unroll
+    for (int o = 0; o < H; ++o) {
+      const C lo = rh ? xp[(3 * H + o) * kDQuadPts] : al[o];
+      const C hi = rh ? xp[(4 * H + o) * kDQuadPts] : xp[(2 * H + o) * kDQuadPts];
+      ar[o] = cadd(lo, hi);
+    }
+  } else {
+#pragma unroll
+    for (int o = 0; o < H; ++o) ar[o] = xp[(rh * H + o) * kDQuadPts];
+#pragma unroll
+    for (int li = 0; li < H; ++li)
+#pragma unroll
+      for (int ri = 0; ri < H; ++ri) ar[ri] = cfma(ar[ri], xl[li], v[li][ri]);
+  }
+#pragma unroll
+  for (int o = 0; o < H; ++o)
+    O[(long long)o * P.ld] = cmk<C>(out[o].x - P.scale * ar[o].x, out[o].y - P.scale * ar[o].y);
+}
+
+// One-sided tile (V_X[Phi] Psi, Poisson solves) of complex vectors, two threads
+// per grid point: half h takes the right orbitals r0 + 4h .. r0 + 4h + 3 and sums
+// over the left ones in turn, four at a time, so that a thread has 16 potentials
+// in flight (a batch is often one tile, and with one thread per point its launch
+// held two blocks per SM with eight potentials in flight per thread): V_X of 61
+// orbitals on 37 bands, 48x40x36: 1.43 -> 1.34 ms.
+constexpr int kDRectPts = 128;   // points per 256-thread block
+template <typename R, long long NGC>
+__device__ __forceinline__ void d_rect(const PointParams<R>& P, const TileDesc& d, long long vbx, int tid) {
+  using C = cplx<R>;
+  const long long NG = NGC ? NGC : P.ng;
+  constexpr int H = kTileMax / 2, U = 4;
+  const int h = (tid >> 5) & 1, n = d.nr - h * H < H ? d.nr - h * H : H;   // right orbitals of this thread
+  const long long g = vbx * kDRectPts + (((tid >> 6) << 5) | (tid & 31));
+  if (g >= NG || n <= 0) return;
+  const C* V = P.S + (long long)(d.slot0 + h * H) * NG + g;
+  const C* X = static_cast<const C*>(P.X) + (long long)d.l0 * P.ld + g;
+  C ar[H];
+#pragma unroll
+  for (int o = 0; o < H; ++o) ar[o] = cmk<C>(R(0), R(0));
+  int li = 0;
+  if (n == H) {
+    for (; li + U <= d.nl; li += U) {
+      C x[U], v[U][H];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        x[u] = X[(long long)(li + u) * P.ld];
+#pragma unroll
+        for (int o = 0; o < H; ++o) v[u][o] = __ldcs(V + (long long)((li + u) * d.nr + o) * NG);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int o = 0; o < H; ++o) ar[o] = cfma(ar[o], x[u], v[u][o]);
+    }
+  }
+  for (; li < d.nl; ++li) {
+    const C x = X[(long long)li * P.ld];
+#pragma unroll
+    for (int o = 0; o < H; ++o)
+      if (o < n) ar[o] = cfma(ar[o], x, __ldcs(V + (long long)(li * d.nr + o) * NG));
+  }
+#pragma unroll
+  for (int o = 0; o < H; ++o)
+    if (o < n) rmw_out<R, false, false>(P.OutY, (long long)(d.r0 + h * H + o) * P.ld + g, ar[o], P.scale);
 }
 
 // Pass D (complex vectors) for point block `vbx` (nthr points) of tile `d`;
@@ -1273,31 +1403,51 @@ pass_c_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
                                                      threadIdx.x);
 }
 
-// Full off-diagonal tiles take two threads per grid point (d_split_off) at
-// four blocks per SM (64 registers): more warps and loads in flight per SM,
-// which measured faster than one thread per point at 2 or 3 blocks per SM
-// (and than streaming the potentials through shared memory with bulk copies).
-// The tiles other than full off-diagonal ones (diagonal, ragged, one-sided):
-// one thread per point, 256 points per block (the grid is sized for 128-point
-// blocks, so the upper half of the blocks has no work). Not inlined, so that
-// its larger register state does not spill into the full-tile path.
+// The other tiles (diagonal, ragged, one-sided ones of real vectors): one thread
+// per point, 256 points per block (beside tiles of smaller blocks in the same
+// batch the upper blocks have no work). Not inlined, so that its larger register
+// state does not spill into the full-tile path.
 template <typename R, bool REAL, long long NGC>
 __device__ __noinline__ void pass_d_other(const PointParams<R>& P, const TileDesc& d) {
   if ((long long)blockIdx.x * 256 >= (NGC ? NGC : P.ng)) return;
   body_d<R, REAL, false, false, NGC>(P, d, blockIdx.x, threadIdx.x, blockDim.x);
 }
 
+// Full off-diagonal tiles: FP32 four threads per grid point (d_quad_off) at three
+// blocks per SM, FP64 two at two. Pass D waits on its loads, so what counts is
+// that a thread issues them all at once: at four blocks (64 registers) the
+// compiler splits them up, and where the spectrum does not fit L2 the pass took
+// 47 us at 64^3 and 158 at 96^3 instead of 39 and 123. Two threads per point at
+// four blocks took 49 and 150; 18.5 -> 16.4 at 48^3, 22.5 -> 18.4 at 32^3 (256 pairs).
+// Points per block of a batch: the fewest that one of its tiles needs.
+template <typename R> int d_points(const Batch& b, bool real) {
+  int pts = 256;
+  for (int t = 0; t < b.ntiles; ++t) {
+    const TileDesc& d = b.t[t];
+    if (d.kind == 0 && d.nl == kTileMax && d.nr == kTileMax) return sizeof(R) == 4 ? kDQuadPts : kDSplitPts;
+    if (d.kind == 2 && !real) pts = kDRectPts;
+  }
+  return pts;
+}
 template <typename R, bool REAL, long long NGC>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
 pass_d_kernel(const __grid_constant__ PointParams<R> P) {
-  __shared__ cplx<R> xch[(kTileMax / 2) * 256];
+  constexpr int B = kTileMax;
+  __shared__ cplx<R> xch[sizeof(R) == 4 ? 5 * (B / 2) * kDQuadPts : (B / 2) * 256];
   griddep_launch();
   griddep_wait();
   const TileDesc d = P.tiles[blockIdx.y];
   if (d.kind == 0 && d.nl == kTileMax && d.nr == kTileMax) {
     if constexpr (REAL) d_split_off_real<R, NGC>(P, d, blockIdx.x, threadIdx.x, reinterpret_cast<R*>(xch));
+    else if constexpr (sizeof(R) == 4) d_quad_off<R, NGC>(P, d, blockIdx.x, threadIdx.x, xch);
     else d_split_off<R, REAL, NGC>(P, d, blockIdx.x, threadIdx.x, xch);
     return;
+  }
+  if constexpr (!REAL) {
+    if (d.kind == 2) {
+      d_rect<R, NGC>(P, d, blockIdx.x, threadIdx.x);
+      return;
+    }
   }
   pass_d_other<R, REAL, NGC>(P, d);
 }
@@ -1553,7 +1703,8 @@ bool launch_point(const PairLaunch& L, const Batch& b, cudaStream_t st) {
   PointParams<R> P;
   fill_point<R>(P, L);
   if (NGC && P.ng != NGC) return false;
-  const dim3 grid((unsigned)((P.ng + kDSplitPts - 1) / kDSplitPts), (unsigned)b.ntiles);
+  const int pts = d_points<R>(b, L.real_io);
+  const dim3 grid((unsigned)((P.ng + pts - 1) / pts), (unsigned)b.ntiles);
   if constexpr (sizeof(R) == 8) {
     if (L.real_io) {
       launch_pdl(!L.no_pdl, pass_d_kernel<R, true, NGC>, grid, dim3(256), 0, st, P);
