@@ -297,7 +297,7 @@ struct WsLayout {
 
 // Split-K partial matrices of a gram product (the tensor-core or CUDA-core one).
 int gram_parts(const ace_plan* p, int na, int nb) {
-  return p->tc ? gram_tc_splits(p->ng, na, nb) : gram_splits(p->ng, na, nb);
+  return p->tc ? gram_tc_splits(p->ng, na, nb) : gram_splits(p->f64, p->ng, na, nb);
 }
 
 // Upper bound on the batches of the one-sided schedule for n_b vectors.
@@ -638,7 +638,7 @@ int issue_xi(ace_plan* p, const void* W, int nk, const double* LinvH, void* Xi, 
     launch_outer_tc(W, nk, LinvH, nk, p->ld, p->ng, 1.0, Xi, c32, p->status, cs);
     return 2;
   }
-  launch_outer(p->f64, p->real, W, nk, LinvH, nk, p->ld, p->ng, 1.0, Xi, cs);
+  launch_outer(p->f64, p->real, W, nk, LinvH, nk, p->ld, p->ng, 1.0, true, Xi, cs);
   return 1;
 }
 
@@ -1385,7 +1385,7 @@ ace_status ace_apply(ace_plan* p, const void* Xi, const void* Psi, int nb, void*
   else launch_gram(p->f64, p->real, Xi, N, Psi, nb, p->ld, p->ng, Wl.part, splits, st);
   launch_gram_reduce(Wl.part, splits, N, nb, p->dv, false, false, Wl.Cm, nullptr, st);
   if (p->tc) launch_outer_tc(Xi, N, Wl.Cm, nb, p->ld, p->ng, -1.0, Y, Wl.part, p->status, st, p->bf16);
-  else launch_outer(p->f64, p->real, Xi, N, Wl.Cm, nb, p->ld, p->ng, -1.0, Y, st);
+  else launch_outer(p->f64, p->real, Xi, N, Wl.Cm, nb, p->ld, p->ng, -1.0, false, Y, st);
   p->launches += p->tc ? 4 : 3;
   return cuda_check("ace_apply");
 }

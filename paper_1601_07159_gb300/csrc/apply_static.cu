@@ -61,7 +61,7 @@ extern "C" ace_status ace_apply_static(ace_plan* p, const void* Xi, const void* 
         ACE_ERR_ARG, ("n_occ * n_b = " + std::to_string((long long)N * nb) +
                       " exceeds the static scratch (max " +
                       std::to_string(ACE_STATIC_SCRATCH_BYTES / (4 * sizeof(double))) + ")").c_str());
-  int splits = ace::gram_splits(ng, N, nb);
+  int splits = ace::gram_splits(f64 != 0, ng, N, nb);
   if ((size_t)splits > fit - 1) splits = (int)(fit - 1);
 
   void* base = nullptr;
@@ -82,7 +82,7 @@ extern "C" ace_status ace_apply_static(ace_plan* p, const void* Xi, const void* 
   cudaStream_t st = (cudaStream_t)stream;
   ace::launch_gram(f64 != 0, real != 0, Xi, N, Psi, nb, ld, ng, part, splits, st);
   ace::launch_gram_reduce(part, splits, N, nb, dv, false, false, Cm, nullptr, st);
-  ace::launch_outer(f64 != 0, real != 0, Xi, N, Cm, nb, ld, ng, -1.0, Y, st);
+  ace::launch_outer(f64 != 0, real != 0, Xi, N, Cm, nb, ld, ng, -1.0, false, Y, st);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)
     return ace_internal_set_error(ACE_ERR_CUDA, (std::string("ace_apply_static: ") + cudaGetErrorString(e)).c_str());

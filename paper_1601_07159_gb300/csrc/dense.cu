@@ -17,29 +17,27 @@ namespace ace {
 
 // ---------------------------------------------------------------- gram
 // part[s][a][b] = sum_{g in chunk s} conj(A[a][g]) B[b][g]   (complex, FP64 out)
-constexpr int GT = 64;   // output tile edge
-constexpr int GK = 16;   // K chunk per shared-memory stage
+constexpr int GT = 64;   // FP32 output tile edge
+constexpr int GK = 16;   // FP32 K chunk per shared-memory stage
 
-template <typename R, bool REAL>
 __global__ void __launch_bounds__(256)
-gram_kernel(const void* __restrict__ A, int na, const void* __restrict__ B, int nb, long long ld,
-            long long ng, double* __restrict__ part, long long chunk) {
-  __shared__ cplx<R> As[GK][GT + 1];
-  __shared__ cplx<R> Bs[GK][GT + 1];
+gram_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B, int nb, long long ld, long long ng,
+            double* __restrict__ part, long long chunk) {
+  __shared__ float2 As[GK][GT + 1];
+  __shared__ float2 Bs[GK][GT + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int a0 = blockIdx.x * GT, b0 = blockIdx.y * GT;
   const long long g_begin = (long long)blockIdx.z * chunk;
   const long long g_end = g_begin + chunk < ng ? g_begin + chunk : ng;
   // this thread's rows a0 + ty + 16 i (i < ni) and columns b0 + tx + 16 j (j < nj)
-  // inside the matrix: small matrices do no work on the tile's padding (on this
-  // part FP64 issue is scarce, and padded warps skip the products entirely)
+  // inside the matrix: small matrices do no work on the tile's padding
   const int ra = na - a0 - ty, rb = nb - b0 - tx;
   const int ni = ra <= 0 ? 0 : (ra + 15) / 16, nj = rb <= 0 ? 0 : (rb + 15) / 16;
-  cplx<R> acc[4][4];
+  float2 acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = cmk<cplx<R>>(R(0), R(0));
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
 
   for (long long g0 = g_begin; g0 < g_end; g0 += GK) {
     // load 64 rows x 16 columns of A and B: 1024 elements each, 4 per thread
@@ -48,18 +46,10 @@ gram_kernel(const void* __restrict__ A, int na, const void* __restrict__ B, int 
       const int idx = threadIdx.x + 256 * e;
       const int row = idx >> 4, col = idx & 15;
       const long long g = g0 + col;
-      cplx<R> va = cmk<cplx<R>>(R(0), R(0)), vb = va;
+      float2 va = make_float2(0.f, 0.f), vb = va;
       if (g < g_end) {
-        if (a0 + row < na) {
-          const long long o = (long long)(a0 + row) * ld + g;
-          if constexpr (REAL) va.x = static_cast<const R*>(A)[o];
-          else va = static_cast<const cplx<R>*>(A)[o];
-        }
-        if (b0 + row < nb) {
-          const long long o = (long long)(b0 + row) * ld + g;
-          if constexpr (REAL) vb.x = static_cast<const R*>(B)[o];
-          else vb = static_cast<const cplx<R>*>(B)[o];
-        }
+        if (a0 + row < na) va = A[(long long)(a0 + row) * ld + g];
+        if (b0 + row < nb) vb = B[(long long)(b0 + row) * ld + g];
       }
       As[col][row] = va;
       Bs[col][row] = vb;
@@ -67,7 +57,7 @@ gram_kernel(const void* __restrict__ A, int na, const void* __restrict__ B, int 
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < GK; ++k) {
-      cplx<R> av[4], bv[4];
+      float2 av[4], bv[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) av[i] = As[k][ty + 16 * i];
 #pragma unroll
@@ -77,7 +67,7 @@ gram_kernel(const void* __restrict__ A, int na, const void* __restrict__ B, int 
         if (i < ni) {
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            if (j < nj) acc[i][j] = cadd(acc[i][j], cmulc(av[i], bv[j]));
+            if (j < nj) acc[i][j] = cadd<false>(acc[i][j], cmulc(av[i], bv[j]));
         }
     }
     __syncthreads();
@@ -97,13 +87,78 @@ gram_kernel(const void* __restrict__ A, int na, const void* __restrict__ B, int 
   }
 }
 
-int gram_splits(long long ng, int na, int nb) {
-  // ~1k-point chunks keep the FP32 partial sums short; small matrices on small
-  // grids take shorter chunks so that the launch still covers one wave of SMs
+// FP64: bound by the FP64 pipe (about 1.7 DFMA per clock and SM), so the tile
+// is chosen for the least padding, not for reuse: 8 x 8 outputs per block, one
+// per thread, with the block's four groups of 64 threads taking every fourth
+// point (their sums meet in a fixed order at the end). Products are fused
+// multiply-adds, and real vectors take one per point instead of a complex
+// product on zeros. 24^3 real, N = 8: 100 -> 6 us; 32^3 complex, N = 27: 693 ->
+// 221 us (64 x 64 tiles, six FP64 operations per complex product before).
+constexpr int GT64 = 8;    // output tile edge
+constexpr int GK64 = 32;   // points per shared-memory stage
+template <bool REAL>
+__global__ void __launch_bounds__(256)
+gram64_kernel(const void* __restrict__ A, int na, const void* __restrict__ B, int nb, long long ld, long long ng,
+              double* __restrict__ part, long long chunk) {
+  __shared__ double2 As[GT64][GK64 + 1];
+  __shared__ double2 Bs[GT64][GK64 + 1];
+  __shared__ double2 red[3][GT64 * GT64];
+  const int kl = threadIdx.x >> 6, o = threadIdx.x & 63, ia = o >> 3, ib = o & 7;
+  const int a0 = blockIdx.x * GT64, b0 = blockIdx.y * GT64;
+  const long long g_begin = (long long)blockIdx.z * chunk;
+  const long long g_end = g_begin + chunk < ng ? g_begin + chunk : ng;
+  const bool work = a0 + (ia & 4) < na;                  // a warp holds four rows
+  const double2 zero = make_double2(0.0, 0.0);
+  auto load = [&](const void* X, int count, int x0, long long g0, int e) {   // element e of the 8 x 32 stage
+    const int row = e / GK64;
+    const long long g = g0 + e % GK64;
+    if (x0 + row >= count || g >= g_end) return zero;
+    const long long off = (long long)(x0 + row) * ld + g;
+    if constexpr (REAL) return make_double2(static_cast<const double*>(X)[off], 0.0);
+    else return static_cast<const double2*>(X)[off];
+  };
+  const int tid = threadIdx.x;
+  double2 va = load(A, na, a0, g_begin, tid), vb = load(B, nb, b0, g_begin, tid);
+  double2 acc = zero;
+  for (long long g0 = g_begin; g0 < g_end; g0 += GK64) {
+    As[tid / GK64][tid % GK64] = va;
+    Bs[tid / GK64][tid % GK64] = vb;
+    __syncthreads();
+    if (g0 + GK64 < g_end) {                             // the next stage's loads run under the products
+      va = load(A, na, a0, g0 + GK64, tid);
+      vb = load(B, nb, b0, g0 + GK64, tid);
+    }
+    if (work) {
+#pragma unroll
+      for (int k = 0; k < GK64 / 4; ++k) {
+        const double2 x = As[ia][4 * k + kl], y = Bs[ib][4 * k + kl];
+        if constexpr (REAL) acc.x = fma(x.x, y.x, acc.x);
+        else acc = cfmac(acc, x, y);
+      }
+    }
+    __syncthreads();
+  }
+  if (kl > 0) red[kl - 1][o] = acc;
+  __syncthreads();
+  if (kl == 0 && a0 + ia < na && b0 + ib < nb) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) acc = cadd(acc, red[q][o]);
+    double2* out = reinterpret_cast<double2*>(part) + (long long)blockIdx.z * na * nb;
+    out[(long long)(a0 + ia) * nb + b0 + ib] = acc;
+  }
+}
+
+int gram_splits(bool f64, long long ng, int na, int nb) {
+  // ~1k-point chunks keep the partial sums short; small matrices on small grids
+  // take shorter chunks so that the launch still covers one wave of SMs (FP64:
+  // four blocks per SM, whose tiles are small)
   long long s = (ng + 1023) / 1024;
-  const long long tiles = (long long)((na + GT - 1) / GT) * ((nb + GT - 1) / GT);
-  const long long wave = tiles > 0 ? (152 + tiles - 1) / tiles : 1;
-  const long long max_s = (ng + GK - 1) / GK;   // at least one K stage per split
+  const int edge = f64 ? GT64 : GT;
+  const long long tiles = (long long)((na + edge - 1) / edge) * ((nb + edge - 1) / edge);
+  const long long blocks = f64 ? 4 * 152 : 152;
+  const long long wave = tiles > 0 ? (blocks + tiles - 1) / tiles : 1;
+  const long long stage = f64 ? GK64 : GK;
+  const long long max_s = (ng + stage - 1) / stage;   // at least one K stage per split
   if (s < wave) s = wave;
   if (s > max_s) s = max_s;
   if (s > 256) s = 256;
@@ -113,14 +168,16 @@ int gram_splits(long long ng, int na, int nb) {
 
 void launch_gram(bool f64, bool real_in, const void* A, int na, const void* B, int nb, long long ld,
                  long long ng, double* part, int splits, cudaStream_t st) {
+  const int edge = f64 ? GT64 : GT, stage = f64 ? GK64 : GK;
   long long chunk = (ng + splits - 1) / splits;
-  chunk = (chunk + GK - 1) / GK * GK;
-  const dim3 grid((na + GT - 1) / GT, (nb + GT - 1) / GT, splits);
+  chunk = (chunk + stage - 1) / stage * stage;
+  const dim3 grid((na + edge - 1) / edge, (nb + edge - 1) / edge, splits);
   if (f64) {
-    if (real_in) gram_kernel<double, true><<<grid, 256, 0, st>>>(A, na, B, nb, ld, ng, part, chunk);
-    else gram_kernel<double, false><<<grid, 256, 0, st>>>(A, na, B, nb, ld, ng, part, chunk);
+    if (real_in) gram64_kernel<true><<<grid, 256, 0, st>>>(A, na, B, nb, ld, ng, part, chunk);
+    else gram64_kernel<false><<<grid, 256, 0, st>>>(A, na, B, nb, ld, ng, part, chunk);
   } else {
-    gram_kernel<float, false><<<grid, 256, 0, st>>>(A, na, B, nb, ld, ng, part, chunk);
+    gram_kernel<<<grid, 256, 0, st>>>(static_cast<const float2*>(A), na, static_cast<const float2*>(B), nb, ld, ng,
+                                      part, chunk);
   }
 }
 
@@ -247,12 +304,11 @@ constexpr int OG = 128;  // g per block
 constexpr int OB = 16;   // b per block
 constexpr int OK = 16;   // k per stage
 
-template <typename R, bool REAL>
 __global__ void __launch_bounds__(256)
-outer_kernel(const void* __restrict__ A, int nk, const double* __restrict__ C, int nb, long long ld,
-             long long ng, double alpha, void* __restrict__ Out) {
-  __shared__ cplx<R> As[OK][OG];
-  __shared__ cplx<R> Cs[OK][OB];
+outer_kernel(const float2* __restrict__ A, int nk, const double* __restrict__ C, int nb, long long ld, long long ng,
+             float alpha, float2* __restrict__ Out) {
+  __shared__ float2 As[OK][OG];
+  __shared__ float2 Cs[OK][OB];
   const int tg = threadIdx.x & 63, tb = threadIdx.x >> 6;   // 64 x 4
   const long long g0 = (long long)blockIdx.x * OG;
   const int b0 = blockIdx.y * OB;
@@ -260,11 +316,11 @@ outer_kernel(const void* __restrict__ A, int nk, const double* __restrict__ C, i
   // warps skip the products)
   const int rbb = nb - b0 - 4 * tb;
   const int nj = rbb <= 0 ? 0 : (rbb < 4 ? rbb : 4);
-  cplx<R> acc[2][4];
+  float2 acc[2][4];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = cmk<cplx<R>>(R(0), R(0));
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
   for (int k0 = 0; k0 < nk; k0 += OK) {
     const int kmax = nk - k0 < OK ? nk - k0 : OK;
 #pragma unroll
@@ -272,20 +328,14 @@ outer_kernel(const void* __restrict__ A, int nk, const double* __restrict__ C, i
       const int idx = threadIdx.x + 256 * e;
       const int kk = idx / OG, gg = idx % OG;
       const long long g = g0 + gg;
-      cplx<R> v = cmk<cplx<R>>(R(0), R(0));
-      if (k0 + kk < nk && g < ng) {
-        const long long o = (long long)(k0 + kk) * ld + g;
-        if constexpr (REAL) v.x = static_cast<const R*>(A)[o];
-        else v = static_cast<const cplx<R>*>(A)[o];
-      }
-      As[kk][gg] = v;
+      As[kk][gg] = (k0 + kk < nk && g < ng) ? A[(long long)(k0 + kk) * ld + g] : make_float2(0.f, 0.f);
     }
     {
       const int kk = threadIdx.x / OB, bb = threadIdx.x % OB;
-      cplx<R> c = cmk<cplx<R>>(R(0), R(0));
+      float2 c = make_float2(0.f, 0.f);
       if (k0 + kk < nk && b0 + bb < nb) {
         const long long o = 2 * ((long long)(k0 + kk) * nb + b0 + bb);
-        c = cmk<cplx<R>>((R)C[o], (R)C[o + 1]);
+        c = make_float2((float)C[o], (float)C[o + 1]);
       }
       Cs[kk][bb] = c;
     }
@@ -293,7 +343,7 @@ outer_kernel(const void* __restrict__ A, int nk, const double* __restrict__ C, i
 #pragma unroll
     for (int k = 0; k < OK; ++k) {
       if (k >= kmax) break;
-      cplx<R> av[2], cv[4];
+      float2 av[2], cv[4];
 #pragma unroll
       for (int i = 0; i < 2; ++i) av[i] = As[k][tg + 64 * i];
 #pragma unroll
@@ -302,7 +352,7 @@ outer_kernel(const void* __restrict__ A, int nk, const double* __restrict__ C, i
       for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (j < nj) acc[i][j] = cadd(acc[i][j], cmul(av[i], cv[j]));
+          if (j < nj) acc[i][j] = cadd<false>(acc[i][j], cmul(av[i], cv[j]));
     }
     __syncthreads();
   }
@@ -313,23 +363,84 @@ outer_kernel(const void* __restrict__ A, int nk, const double* __restrict__ C, i
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int b = b0 + tb * 4 + j;
-      if (b >= nb) continue;
-      const long long o = (long long)b * ld + g;
-      if constexpr (REAL) static_cast<R*>(Out)[o] = (R)alpha * acc[i][j].x;
-      else static_cast<cplx<R>*>(Out)[o] = cscale(acc[i][j], (R)alpha);
+      if (b < nb) Out[(long long)b * ld + g] = cscale(acc[i][j], alpha);
     }
   }
 }
 
-void launch_outer(bool f64, bool real_io, const void* A, int nk, const double* C, int nb,
-                  long long ld, long long ng, double alpha, void* Out, cudaStream_t st) {
-  const dim3 grid((unsigned)((ng + OG - 1) / OG), (nb + OB - 1) / OB);
-  if (f64) {
-    if (real_io) outer_kernel<double, true><<<grid, 256, 0, st>>>(A, nk, C, nb, ld, ng, alpha, Out);
-    else outer_kernel<double, false><<<grid, 256, 0, st>>>(A, nk, C, nb, ld, ng, alpha, Out);
-  } else {
-    outer_kernel<float, false><<<grid, 256, 0, st>>>(A, nk, C, nb, ld, ng, alpha, Out);
+// FP64, bound by the FP64 pipe as the gram product: 64 points x 16 columns per
+// block, one point x 4 columns per thread, fused multiply-adds (real vectors:
+// one per term, C's real part), and with `upper` (C = L^{-*}, zero below the
+// diagonal) only the terms k <= b of each four columns. 24^3 real, N = 8: 17 ->
+// 6 us; 32^3 complex, N = 27: 378 -> 113 us.
+constexpr int OG64 = 64;
+template <bool REAL>
+__global__ void __launch_bounds__(256)
+outer64_kernel(const void* __restrict__ A, int nk, const double2* __restrict__ C, int nb, long long ld, long long ng,
+               double alpha, int upper, void* __restrict__ Out) {
+  __shared__ double2 As[OK][OG64];
+  __shared__ double2 Cs[OK][OB];
+  const int tg = threadIdx.x & 63, tb = threadIdx.x >> 6;   // 64 x 4
+  const long long g0 = (long long)blockIdx.x * OG64, g = g0 + tg;
+  const int b0 = blockIdx.y * OB, bt = b0 + 4 * tb;
+  const int nj = nb - bt < 4 ? nb - bt : 4;
+  const int kend = upper && b0 + OB < nk ? b0 + OB : nk;                  // of the block
+  const int kthr = nj <= 0 ? 0 : upper && bt + 4 < nk ? bt + 4 : nk;      // of this thread (uniform in a warp)
+  double2 acc[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) acc[j] = make_double2(0.0, 0.0);
+  for (int k0 = 0; k0 < kend; k0 += OK) {
+#pragma unroll
+    for (int e = 0; e < (OK * OG64) / 256; ++e) {
+      const int kk = (threadIdx.x >> 6) + 4 * e;
+      double2 v = make_double2(0.0, 0.0);
+      if (k0 + kk < kend && g < ng) {
+        const long long o = (long long)(k0 + kk) * ld + g;
+        if constexpr (REAL) v.x = static_cast<const double*>(A)[o];
+        else v = static_cast<const double2*>(A)[o];
+      }
+      As[kk][tg] = v;
+    }
+    {
+      const int kk = threadIdx.x / OB, bb = threadIdx.x % OB;
+      Cs[kk][bb] = (k0 + kk < kend && b0 + bb < nb) ? C[(long long)(k0 + kk) * nb + b0 + bb] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    const int km = kthr - k0 < OK ? kthr - k0 : OK;
+    for (int k = 0; k < km; ++k) {
+      const double2 x = As[k][tg];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j < nj) {
+          if constexpr (REAL) acc[j].x = fma(x.x, Cs[k][4 * tb + j].x, acc[j].x);
+          else acc[j] = cfma(acc[j], x, Cs[k][4 * tb + j]);
+        }
+      }
+    }
+    __syncthreads();
   }
+  if (g >= ng) return;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (j >= nj) continue;
+    const long long o = (long long)(bt + j) * ld + g;
+    if constexpr (REAL) static_cast<double*>(Out)[o] = alpha * acc[j].x;
+    else static_cast<double2*>(Out)[o] = cscale(acc[j], alpha);
+  }
+}
+
+void launch_outer(bool f64, bool real_io, const void* A, int nk, const double* C, int nb,
+                  long long ld, long long ng, double alpha, bool upper, void* Out, cudaStream_t st) {
+  if (!f64) {
+    const dim3 grid((unsigned)((ng + OG - 1) / OG), (nb + OB - 1) / OB);
+    outer_kernel<<<grid, 256, 0, st>>>(static_cast<const float2*>(A), nk, C, nb, ld, ng, (float)alpha,
+                                       static_cast<float2*>(Out));
+    return;
+  }
+  const dim3 grid((unsigned)((ng + OG64 - 1) / OG64), (nb + OB - 1) / OB);
+  const double2* c = reinterpret_cast<const double2*>(C);
+  if (real_io) outer64_kernel<true><<<grid, 256, 0, st>>>(A, nk, c, nb, ld, ng, alpha, upper, Out);
+  else outer64_kernel<false><<<grid, 256, 0, st>>>(A, nk, c, nb, ld, ng, alpha, upper, Out);
 }
 
 // Xi = W L^{-*} with FP64 arithmetic from FP32 vectors (the plain FP64 form
