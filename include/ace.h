@@ -122,8 +122,9 @@ typedef struct {
                         vectors, two for ACE_DTYPE_R64 (real and imaginary parts) */
   int tile;          /* orbitals per pair tile, 1..8 (0 = default 8) */
   int lanes;         /* concurrent batch streams inside one call with
-                        ACE_FLAG_NO_OVERLAP, 1..8 (0 = default 2; at least 2
-                        otherwise); the pair scratch is lanes * max_pairs slots */
+                        ACE_FLAG_NO_OVERLAP, 1..8 (0 = default 2; without the flag
+                        1 for C64, at least 2 for FP64); the pair scratch is
+                        lanes * max_pairs slots */
   int flags;         /* ACE_FLAG_* */
 } ace_desc;
 
@@ -144,11 +145,13 @@ typedef struct {
 /* ACE_DTYPE_C64: the same as prec = ACE_PREC_FP32 (M, Xi and the apply in FP32
  * on CUDA cores). */
 #define ACE_FLAG_SIMT_GEMM 8
-/* By default, graph mode issues pass A of every pair batch on one stream and
- * passes B-D on a second, so that pass A of batch k+1 (which waits for pass C of
- * batch k) overlaps pass D of batch k; the scratch holds two batches (lanes is
- * raised to at least 2). This flag turns that off: the batches of a round are
- * then spread over `lanes` streams instead. Results are bitwise the same. */
+/* By default, graph mode runs the passes of C64 plans as one chain on one stream
+ * (programmatic dependent launches; the scratch holds one batch, or `lanes`), and
+ * issues pass A of every pair batch of FP64 plans on one stream and passes B-D on
+ * a second, so that pass A of batch k+1 (which waits for pass C of batch k)
+ * overlaps pass D of batch k (the scratch holds two batches, lanes is raised to at
+ * least 2). This flag turns that off: the batches of a round are then spread over
+ * `lanes` streams instead. Results are bitwise the same. */
 #define ACE_FLAG_NO_OVERLAP 16
 /* Radix order of the line transforms (ACE_DTYPE_C64 plans): by default a
  * transform of length n takes a radix 4 first, then 2, 3, 5; with this flag it

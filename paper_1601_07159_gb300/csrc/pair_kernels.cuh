@@ -122,11 +122,16 @@ template <typename R> struct PointParams {
 };
 
 // Programmatic dependent launch (four-kernel mode): every pass is launched with
-// programmatic stream serialisation, so its blocks can be scheduled while the
-// previous pass drains; griddep_wait() blocks until the previous grid has
-// completed and its writes are visible. Without the attribute both are no-ops.
+// programmatic stream serialisation, so its blocks take the slots that the
+// previous pass's last blocks leave; griddep_wait() blocks until the previous
+// grid has completed and its writes are visible (a no-op without the attribute).
+// No pass triggers its dependents itself (griddepcontrol.launch_dependents): a
+// trigger at the start of the blocks let the next pass's blocks pile up on the
+// few SMs with free slots, where they waited and then ran, while the other SMs
+// idled. Passes A-D of one 64-pair tile, trigger at the start -> at block exit:
+// 96^3 715 -> 646 us, 64^3 183 -> 170, 48^3 58.6 -> 56, 256 pairs of 16^3 16 -> 12
+// (without programmatic launch 656, 181, 66, 21).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename Kern, typename... Args>
 inline void launch_pdl(bool pdl, Kern kern, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
@@ -958,7 +963,6 @@ template <typename R, int NX, int NY, bool REAL>
 __global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), plane_blocks<R, NX, NY>())
 pass_a_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  griddep_launch();
   body_a<R, NX, NY, REAL, false, plane_items<R, NX, NY>(), true, kLine2<R, NX, NY>>(
       P, P.tiles, P.ntiles, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x, threadIdx.x);
 }
@@ -1047,7 +1051,6 @@ pass_b_split_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
   constexpr int N = NZ, M = N / 2, H = N / 4;
   static_assert(N % 4 == 0, "the split pass B halves a pencil twice");
   __shared__ double red[8];
-  griddep_launch();
   griddep_wait();
   const PencilGeom<R, NZ, CUBE> G(P);
   const int nxy = G.nxy;
@@ -1142,7 +1145,6 @@ pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   static_assert(kSplitWarps<NX, NY>, "a line's lanes share a warp");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  griddep_launch();
   const int tid = threadIdx.x, q = split_line(tid), h = split_half(tid);
   const long long item = blockIdx.x;                      // one (pair, z) plane per block, z-major:
   const int z = (int)(item / P.npairs), p = (int)(item % P.npairs);   // pairs sharing a plane run together
@@ -1202,7 +1204,6 @@ pass_c_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   static_assert(kSplitWarps<NX, NY>, "a line's lanes share a warp");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  griddep_launch();
   griddep_wait();
   const int tid = threadIdx.x, q = split_line(tid), h = split_half(tid);
   const long long item = blockIdx.x;
@@ -1314,7 +1315,6 @@ pass_b_quad_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
   static_assert(M % 4 == 0, "M / 4 frequencies per thread");
   __shared__ C buf[N * LP];                                // [phase h, k][pencil]
   __shared__ double red[4];
-  griddep_launch();
   griddep_wait();
   const PencilGeom<R, NZ, CUBE> G(P);
   const int nxy = G.nxy;
@@ -1387,7 +1387,6 @@ template <typename R, int NZ, bool CUBE>
 __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 1 : 2)
 pass_b_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
   __shared__ double red[32];
-  griddep_launch();
   griddep_wait();
   body_b<R, NZ, false, CUBE>(P, P.tiles, P.ntiles, P.npairs, mode, blockIdx.x, threadIdx.x, blockDim.x, red,
                              mode != 0 ? P.Epart + blockIdx.x : nullptr);
@@ -1397,7 +1396,6 @@ template <typename R, int NX, int NY>
 __global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), plane_blocks<R, NX, NY>())
 pass_c_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  griddep_launch();
   griddep_wait();
   body_c<R, NX, NY, false, plane_items<R, NX, NY>(), kLine2<R, NX, NY>>(P, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x,
                                                      threadIdx.x);
@@ -1434,7 +1432,6 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
 pass_d_kernel(const __grid_constant__ PointParams<R> P) {
   constexpr int B = kTileMax;
   __shared__ cplx<R> xch[sizeof(R) == 4 ? 5 * (B / 2) * kDQuadPts : (B / 2) * 256];
-  griddep_launch();
   griddep_wait();
   const TileDesc d = P.tiles[blockIdx.y];
   if (d.kind == 0 && d.nl == kTileMax && d.nr == kTileMax) {
