@@ -124,6 +124,26 @@ __device__ __forceinline__ cplx<R> twiddle_value(int e, const TwTable<R, NTOP>& 
   return INV ? cmk<cplx<R>>(w.x, -w.y) : w;
 }
 
+// s = a + w b and d = a - w b with w = w_N^e (conjugated for the inverse), as six
+// fused operations: s by four, d = 2 a - s by two, instead of four for the
+// product and four sums. The FP64 passes are bound by the FP64 pipe, so they
+// gain what they save: passes A, B, C of a 64-pair tile 581, 488, 518 -> 545, 452,
+// 483 us at 48^3 (FP32 pair additions are one packed instruction each).
+template <int N, int NTOP, bool INV, typename R>
+__device__ __forceinline__ void tw_sum_diff(cplx<R> a, cplx<R> b, int e, const TwTable<R, NTOP>& tw, cplx<R>& s,
+                                            cplx<R>& d) {
+  e %= N;
+  if ((4 * e) % N == 0) {
+    const cplx<R> t = twiddle<N, NTOP, INV, R>(b, e, tw);
+    s = cadd(a, t);
+    d = csub(a, t);
+    return;
+  }
+  const cplx<R> w = twiddle_value<N, NTOP, INV, R>(e, tw);
+  s = cmk<cplx<R>>(fma(-w.y, b.y, fma(w.x, b.x, a.x)), fma(w.y, b.x, fma(w.x, b.y, a.y)));
+  d = cmk<cplx<R>>(fma(R(2), a.x, -s.x), fma(R(2), a.y, -s.y));
+}
+
 template <int N> __host__ __device__ constexpr int first_radix() {
   if constexpr (ACE_RADIX_ORDER == 1 && N % 3 == 0 && N != 3) return 3;
   if constexpr (ACE_RADIX_ORDER == 1 && N % 5 == 0 && N != 5) return 5;
@@ -209,9 +229,24 @@ __device__ __forceinline__ void dft(cplx<R> (&a)[N], const TwTable<R, NTOP>& tw)
 #pragma unroll
     for (int k = 0; k < M; ++k) {
       cplx<R> t[RX];
+      if constexpr (sizeof(R) == 8 && (RX == 2 || RX == 4)) {   // FP64: twiddles fused into the butterfly
+        if constexpr (RX == 2) {
+          tw_sum_diff<N, NTOP, INV, R>(sub[0][k], sub[1][k], k, tw, t[0], t[1]);
+        } else {
+          cplx<R> s02, d02, s13, d13;
+          tw_sum_diff<N, NTOP, INV, R>(sub[0][k], sub[2][k], 2 * k, tw, s02, d02);
+          tw_sum_diff<N, NTOP, INV, R>(twiddle<N, NTOP, INV, R>(sub[1][k], k, tw), sub[3][k], 3 * k, tw, s13, d13);
+          d13 = rot_q<INV>(d13);
+          t[0] = cadd(s02, s13);
+          t[2] = csub(s02, s13);
+          t[1] = cadd(d02, d13);
+          t[3] = csub(d02, d13);
+        }
+      } else {
 #pragma unroll
-      for (int r = 0; r < RX; ++r) t[r] = twiddle<N, NTOP, INV, R>(sub[r][k], r * k, tw);
-      dft<RX, NTOP, INV, R, PK>(t, tw);
+        for (int r = 0; r < RX; ++r) t[r] = twiddle<N, NTOP, INV, R>(sub[r][k], r * k, tw);
+        dft<RX, NTOP, INV, R, PK>(t, tw);
+      }
 #pragma unroll
       for (int q = 0; q < RX; ++q) a[k + M * q] = t[q];
     }

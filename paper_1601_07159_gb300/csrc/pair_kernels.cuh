@@ -247,16 +247,15 @@ template <typename R, int NZ, bool CUBE> struct PencilGeom {
 
 template <int NX, int NY> constexpr int kMaxLine = NX > NY ? NX : NY;
 
-// Items (pair, z-plane) per CTA of the whole-line plane kernels. FP32: about 128
+// Items (pair, z-plane) per CTA of the whole-line plane kernels: about 128
 // threads (two planes of 48 or 64, five of 24), so that several independent
 // blocks share an SM and one block's loads run under another's transforms;
 // about 256 threads left one or two blocks per SM that loaded, transformed and
 // stored together (a 64-pair tile, passes A + C: 24^3 8.3 -> 7.3, 32^3 6.0 ->
-// 5.0, 36^3 7.3 -> 6.6 ps per pair point). FP64: about 256 threads, <= 96 KB.
+// 5.0, 36^3 7.3 -> 6.6 ps per pair point; FP64 24^3 242 -> 170). At most 96 KB.
 template <typename R, int NX, int NY> __host__ __device__ constexpr int plane_items() {
   constexpr int ML = kMaxLine<NX, NY>;
-  constexpr int want = sizeof(R) == 4 ? 128 : 256;
-  constexpr int by_threads = (want / ML) > 0 ? (want / ML) : 1;
+    constexpr int by_threads = (128 / ML) > 0 ? (128 / ML) : 1;
   constexpr int by_smem = (96 * 1024) / (NY * (NX + 1) * (int)sizeof(cplx<R>));
   constexpr int v = by_threads < by_smem ? by_threads : by_smem;
   return v > 0 ? v : 1;
@@ -1381,10 +1380,13 @@ pass_b_quad_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
   }
 }
 
-// FP64 pencils of 48 hold 96 doubles: one block per SM (two would cap a thread
-// at 128 registers and spill about 3 KB).
+// Blocks of 64 pencils, one per thread, so that a small call (one density on 48^3
+// has 2304 pencils) spreads over the chip: nine blocks of 256 did not. 512
+// threads per SM for FP32; FP64 pencils of 48 hold 96 doubles, so 256 (more would
+// cap a thread at 128 registers and spill about 3 KB).
+constexpr int kPencilThreads = 64;
 template <typename R, int NZ, bool CUBE>
-__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 1 : 2)
+__global__ void __launch_bounds__(kPencilThreads, (sizeof(R) == 8 ? 256 : 512) / kPencilThreads)
 pass_b_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
   __shared__ double red[32];
   griddep_wait();
@@ -1678,8 +1680,8 @@ void launch_pencil_as(const PencilParams<R, NZ>& P, const PairLaunch& L, long lo
     const unsigned grid = (unsigned)((pencils + kBSplitPencils - 1) / kBSplitPencils);
     launch_pdl(!L.no_pdl, pass_b_split_kernel<R, NZ, CUBE>, dim3(grid), dim3(256), 0, st, P, L.mode);
   } else {
-    const unsigned grid = (unsigned)((pencils + 255) / 256);
-    launch_pdl(!L.no_pdl, pass_b_kernel<R, NZ, CUBE>, dim3(grid), dim3(256), 0, st, P, L.mode);
+    const unsigned grid = (unsigned)((pencils + kPencilThreads - 1) / kPencilThreads);
+    launch_pdl(!L.no_pdl, pass_b_kernel<R, NZ, CUBE>, dim3(grid), dim3(kPencilThreads), 0, st, P, L.mode);
   }
 }
 template <typename R, int NZ>
