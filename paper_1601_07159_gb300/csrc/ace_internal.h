@@ -43,10 +43,12 @@ __host__ __device__ inline int tile_slots(const TileDesc& d, bool real) {
 struct PairLaunch {
   int nx, ny, nz;        // grid points along x, y, z
   long long ld;          // elements from one vector to the next (>= n_x n_y n_z)
-  const void* X;         // l-side vectors (phi)
+  const void* X;         // l-side vectors (phi); null: the constant orbital 1 (not in the engine)
   const void* Y;         // r-side vectors (phi or psi)
   void* OutX;            // accumulators for the l side (symmetric tiles)
   void* OutY;            // accumulators for the r side
+  void* V;               // nullable: pass C writes the potentials to these vectors (by r) instead of S
+  int* clear;            // nullable: status word reset by pass A
   void* S;               // spectrum scratch, max_pairs * N_g complex
   const void* Kt;        // kernel table K(G) alpha / N_g, folded [kz][kx][ky] over 0..n/2 per axis
   double* Epart;         // per-block energy partials (nullable)

@@ -81,10 +81,16 @@ template <typename R, int N> struct PlaneTw<R, N, N> {
   }
 };
 
-// Passes A and C: the pair's vectors (pass A), the scratch, nz z-planes per pair.
+// Passes A and C: the pair's vectors, the scratch, nz z-planes per pair. Poisson
+// solves (instances POIS) have the constant orbital 1 for X, which pass A leaves
+// out, and their potentials are the result: pass C writes slot (l, r)'s to vector
+// r of V instead of the scratch. (As run-time cases these cost pass C 10 % at 96^3.)
 template <typename R, int NX, int NY> struct PlaneParams {
   const void* X;
   const void* Y;
+  void* V;
+  int* clear;              // status word that the first block of pass A resets (nullable)
+  int packed;              // real vectors: two pairs per slot
   cplx<R>* S;
   long long ld;
   int nz;
@@ -291,7 +297,7 @@ __device__ __forceinline__ void line_dft(cplx<R> (&a)[N], const TwTable<R, N>& t
   else dft<N, N, INV, R>(a, tw);
 }
 // Pass A on virtual block `vb` (IPB plane items, thread tid = ty * max(NX, NY) + tx).
-template <typename R, int NX, int NY, bool REAL, bool COH, int IPB, bool PDL, bool LINE2>
+template <typename R, int NX, int NY, bool REAL, bool COH, int IPB, bool PDL, bool LINE2, bool POIS>
 __device__ __forceinline__ void body_a(const PlaneParams<R, NX, NY>& P, const TileDesc* tiles, int ntiles,
                                        int npairs, cplx<R>* smem, long long vb, int tid) {
   constexpr int ML = kMaxLine<NX, NY>;
@@ -317,13 +323,13 @@ __device__ __forceinline__ void body_a(const PlaneParams<R, NX, NY>& P, const Ti
       const long long y2o = (long long)(two ? r2 : r) * P.ld + (long long)z * NX * NY + tx;
 #pragma unroll
       for (int y = 0; y < NY; ++y) {
-        const R xv = Xr[xo + y * NX];
+        const R xv = POIS ? R(1) : Xr[xo + y * NX];
         a[y] = cmk<cplx<R>>(xv * Yr[yo + y * NX], two ? xv * Yr[y2o + y * NX] : R(0));
       }
     } else {
 #pragma unroll
       for (int y = 0; y < NY; ++y) {
-        const cplx<R> xv = load_vec<R, REAL>(P.X, xo + y * NX);
+        const cplx<R> xv = POIS ? cmk<cplx<R>>(R(1), R(0)) : load_vec<R, REAL>(P.X, xo + y * NX);
         const cplx<R> yv = load_vec<R, REAL>(P.Y, yo + y * NX);
         a[y] = cmulc(xv, yv);                 // conj(x_l) * y_r
       }
@@ -338,7 +344,10 @@ __device__ __forceinline__ void body_a(const PlaneParams<R, NX, NY>& P, const Ti
 #pragma unroll
     for (int x = 0; x < NX; ++x) b[x] = buf[tx * (NX + 1) + x];
     line_dft<NX, false, LINE2, R>(b, P.tw.tx());   // along x, row ky = tx
-    if constexpr (PDL) griddep_wait();        // the previous batch's pass D still reads S
+    if constexpr (PDL) {
+      griddep_wait();                         // the previous batch's pass D still reads S
+      if (P.clear && vb == 0 && tid == 0) P.clear[0] = P.clear[1] = 0;
+    }
     cplx<R>* out = P.S + ((long long)p * P.nz + z) * NX * NY + tx;
 #pragma unroll
     for (int kx = 0; kx < NX; ++kx) stx<COH>(out + kx * NY, b[kx]);
@@ -392,8 +401,37 @@ __device__ __forceinline__ void body_b(const PencilParams<R, NZ>& P, const TileD
   }
 }
 
+// Where pass C leaves plane z of slot p: point i of the plane goes through store(i, v).
+template <typename R, int NX, int NY, bool COH, bool POIS> struct PlaneOut {
+  cplx<R>* c = nullptr;          // complex destination (the scratch or a vector of V)
+  R *re = nullptr, *im = nullptr;   // real vectors of V (packed slots; im null: none)
+  __device__ __forceinline__ PlaneOut(const PlaneParams<R, NX, NY>& P, int p, int z, cplx<R>* plane) {
+    c = plane;
+    if constexpr (POIS) {
+      int l, r, r2 = -1;
+      if (sizeof(R) == 8 && P.packed) {
+        decode_slot_real(P.tiles, P.ntiles, p, l, r, r2);
+        R* V = static_cast<R*>(P.V) + (long long)z * NX * NY;
+        re = V + (long long)r * P.ld;
+        im = r2 >= 0 ? V + (long long)r2 * P.ld : nullptr;
+      } else {
+        decode_pair(P.tiles, P.ntiles, p, l, r);
+        c = static_cast<cplx<R>*>(P.V) + (long long)r * P.ld + (long long)z * NX * NY;
+      }
+    }
+  }
+  __device__ __forceinline__ void store(int i, cplx<R> v) const {
+    if (sizeof(R) == 8 && POIS && re) {
+      re[i] = v.x;
+      if (im) im[i] = v.y;
+    } else {
+      stx<COH>(c + i, v);
+    }
+  }
+};
+
 // Pass C on virtual block `vb` (IPB plane items).
-template <typename R, int NX, int NY, bool COH, int IPB, bool LINE2>
+template <typename R, int NX, int NY, bool COH, int IPB, bool LINE2, bool POIS>
 __device__ __forceinline__ void body_c(const PlaneParams<R, NX, NY>& P, int npairs, cplx<R>* smem, long long vb,
                                        int tid) {
   constexpr int ML = kMaxLine<NX, NY>;
@@ -402,9 +440,10 @@ __device__ __forceinline__ void body_c(const PlaneParams<R, NX, NY>& P, int npai
   const long long item = vb * IPB + ty;
   const bool active = ty < IPB && item < (long long)npairs * P.nz;
   cplx<R>* plane = nullptr;
+  int p = 0, z = 0;
   if (active) {
-    const int p = (int)(item / P.nz);
-    const int z = (int)(item % P.nz);
+    p = (int)(item / P.nz);
+    z = (int)(item % P.nz);
     plane = P.S + ((long long)p * P.nz + z) * NX * NY;
   }
   if (active && tx < NY) {
@@ -421,8 +460,9 @@ __device__ __forceinline__ void body_c(const PlaneParams<R, NX, NY>& P, int npai
 #pragma unroll
     for (int ky = 0; ky < NY; ++ky) a[ky] = buf[ky * (NX + 1) + tx];  // column x = tx
     line_dft<NY, true, LINE2, R>(a, P.tw.ty());                       // inverse along y
+    const PlaneOut<R, NX, NY, COH, POIS> out(P, p, z, plane);
 #pragma unroll
-    for (int y = 0; y < NY; ++y) stx<COH>(plane + y * NX + tx, a[y]);
+    for (int y = 0; y < NY; ++y) out.store(y * NX + tx, a[y]);
   }
 }
 
@@ -958,11 +998,11 @@ __device__ __forceinline__ void body_d(const PointParams<R>& P, const TileDesc& 
 }
 
 // ---------------------------------------------------------------- four-kernel mode
-template <typename R, int NX, int NY, bool REAL>
+template <typename R, int NX, int NY, bool REAL, bool POIS>
 __global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), plane_blocks<R, NX, NY>())
 pass_a_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  body_a<R, NX, NY, REAL, false, plane_items<R, NX, NY>(), true, kLine2<R, NX, NY>>(
+  body_a<R, NX, NY, REAL, false, plane_items<R, NX, NY>(), true, kLine2<R, NX, NY>, POIS>(
       P, P.tiles, P.ntiles, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x, threadIdx.x);
 }
 
@@ -1137,7 +1177,7 @@ template <int N> __device__ __forceinline__ int split_index(int j, int h) {
 // nothing, so every lane of a warp takes part in the shuffles. Scalar additions:
 // with packed ones the 96-point passes measured 212 -> 207 (A) but 188 -> 207 us
 // (C) per 64-pair tile.
-template <typename R, int NX, int NY, bool REAL>
+template <typename R, int NX, int NY, bool REAL, bool POIS>
 __global__ void __launch_bounds__(2 * kMaxLine<NX, NY>, kSplitBlocks<R, NX, NY>)
 pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   using C = cplx<R>;
@@ -1165,14 +1205,16 @@ pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         const int yy = 2 * m + h;
-        const R xv = act ? Xr[xo + yy * NX] : R(0);
+        const R xv = !act ? R(0) : POIS ? R(1) : Xr[xo + yy * NX];
         a[m] = act ? cmk<C>(xv * Yr[yo + yy * NX], two ? xv * Yr[y2o + yy * NX] : R(0)) : zero;
       }
     } else {
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         const int yy = 2 * m + h;
-        a[m] = act ? cmulc(load_vec<R, REAL>(P.X, xo + yy * NX), load_vec<R, REAL>(P.Y, yo + yy * NX)) : zero;
+        a[m] = act ? cmulc(POIS ? cmk<C>(R(1), R(0)) : load_vec<R, REAL>(P.X, xo + yy * NX),
+                           load_vec<R, REAL>(P.Y, yo + yy * NX))
+                   : zero;
       }
     }
     dft<M, NY, false, R, false>(a, P.tw.ty());            // along y
@@ -1189,6 +1231,7 @@ pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
     for (int m = 0; m < M; ++m) a[m] = act ? buf[q * (NX + 1) + 2 * m + h] : zero;
     dft<M, NX, false, R, false>(a, P.tw.tx());            // along x
     griddep_wait();                                        // the previous batch's pass D still reads S
+    if (P.clear && blockIdx.x == 0 && tid == 0) P.clear[0] = P.clear[1] = 0;
     C* out = P.S + ((long long)p * P.nz + z) * NX * NY + q;
     split_combine<NX, false, R>(a, h, P.tw.tx(), [&](int j, C v) {
       if (act) out[(long long)split_index<NX>(j, h) * NY] = v;
@@ -1196,7 +1239,7 @@ pass_a_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   }
 }
 
-template <typename R, int NX, int NY>
+template <typename R, int NX, int NY, bool POIS>
 __global__ void __launch_bounds__(2 * kMaxLine<NX, NY>, kSplitBlocks<R, NX, NY>)
 pass_c_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   using C = cplx<R>;
@@ -1228,8 +1271,9 @@ pass_c_split_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
 #pragma unroll
     for (int m = 0; m < M; ++m) a[m] = act ? buf[(2 * m + h) * (NX + 1) + q] : zero;
     dft<M, NY, true, R, false>(a, P.tw.ty());
+    const PlaneOut<R, NX, NY, false, POIS> out(P, p, z, plane);
     split_combine<NY, true, R>(a, h, P.tw.ty(), [&](int j, C v) {
-      if (act) plane[(long long)split_index<NY>(j, h) * NX + q] = v;
+      if (act) out.store(split_index<NY>(j, h) * NX + q, v);
     });
   }
 }
@@ -1394,12 +1438,12 @@ pass_b_kernel(const __grid_constant__ PencilParams<R, NZ> P, int mode) {
                              mode != 0 ? P.Epart + blockIdx.x : nullptr);
 }
 
-template <typename R, int NX, int NY>
+template <typename R, int NX, int NY, bool POIS>
 __global__ void __launch_bounds__(kMaxLine<NX, NY> * plane_items<R, NX, NY>(), plane_blocks<R, NX, NY>())
 pass_c_kernel(const __grid_constant__ PlaneParams<R, NX, NY> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   griddep_wait();
-  body_c<R, NX, NY, false, plane_items<R, NX, NY>(), kLine2<R, NX, NY>>(P, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x,
+  body_c<R, NX, NY, false, plane_items<R, NX, NY>(), kLine2<R, NX, NY>, POIS>(P, P.npairs, reinterpret_cast<cplx<R>*>(smem_raw), blockIdx.x,
                                                      threadIdx.x);
 }
 
@@ -1542,12 +1586,12 @@ pair_engine_kernel(const __grid_constant__ EngineParams<R, N> E) {
     const EngineBatch& b = E.batches[k];
     const TileDesc* tiles = E.pl.tiles + b.toff;
     if (pass == 0) {
-      body_a<R, N, N, REAL, true, IPB, false, false>(E.pl, tiles, b.ntiles, b.npairs, smem, loc, tid);
+      body_a<R, N, N, REAL, true, IPB, false, false, false>(E.pl, tiles, b.ntiles, b.npairs, smem, loc, tid);
     } else if (pass == 1) {
       body_b<R, N, true, true>(E.pe, tiles, b.ntiles, b.npairs, E.mode, loc, tid, kEngineThreads, red,
                                E.mode != 0 ? E.pe.Epart + loc : nullptr);
     } else if (pass == 2) {
-      body_c<R, N, N, true, IPB, false>(E.pl, b.npairs, smem, loc, tid);
+      body_c<R, N, N, true, IPB, false, false>(E.pl, b.npairs, smem, loc, tid);
     } else {
       const long long nvb = ((long long)N * N * N + kEngineThreads - 1) / kEngineThreads;
       const TileDesc d = tiles[loc / nvb];
@@ -1566,6 +1610,9 @@ template <typename R, int NX, int NY>
 void fill_plane(PlaneParams<R, NX, NY>& P, const PairLaunch& L, const Batch& b) {
   P.X = L.X;
   P.Y = L.Y;
+  P.V = L.V;
+  P.clear = L.clear;
+  P.packed = L.real_io ? 1 : 0;
   P.S = static_cast<cplx<R>*>(L.S);
   P.ld = L.ld;
   P.nz = L.nz;
@@ -1611,62 +1658,45 @@ void fill_point(PointParams<R>& P, const PairLaunch& L) {
 // Pass A (pass == 0) or C (pass == 2) of one batch, or (prepare_only) the
 // kernels' shared-memory attributes, set once at plan creation on the plan's
 // device, never during stream capture.
+template <typename R, int NX, int NY, bool POIS>
+void launch_plane_as(const PairLaunch& L, const Batch& b, int pass, cudaStream_t st) {
+  constexpr bool F64 = sizeof(R) == 8, SPLIT = kSplitPlanes<R, NX, NY>;
+  constexpr int IPB = SPLIT ? 1 : plane_items<R, NX, NY>();
+  constexpr size_t smem = SPLIT ? kSplitSmem<R, NX, NY> : (size_t)IPB * NY * (NX + 1) * sizeof(cplx<R>);
+  PlaneParams<R, NX, NY> P;
+  if (!L.prepare_only) fill_plane<R, NX, NY>(P, L, b);
+  const long long items = (long long)b.npairs * L.nz;
+  const dim3 grid((unsigned)((items + IPB - 1) / IPB)), blk(kMaxLine<NX, NY> * (SPLIT ? 2 : IPB));
+  auto run = [&](auto kern) {
+    if (L.prepare_only) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    } else {
+      launch_pdl(!L.no_pdl, kern, grid, blk, smem, st, P);
+    }
+  };
+  if constexpr (SPLIT) {
+    if (pass == 2) run(pass_c_split_kernel<R, NX, NY, POIS>);
+    else if (F64 && L.real_io) run(pass_a_split_kernel<R, NX, NY, F64, POIS>);
+    else run(pass_a_split_kernel<R, NX, NY, false, POIS>);
+  } else {
+    if (pass == 2) run(pass_c_kernel<R, NX, NY, POIS>);
+    else if (F64 && L.real_io) run(pass_a_kernel<R, NX, NY, F64, POIS>);
+    else run(pass_a_kernel<R, NX, NY, false, POIS>);
+  }
+}
 template <typename R, int NX, int NY>
 bool launch_plane(const PairLaunch& L, const Batch& b, int pass, cudaStream_t st) {
-  constexpr int IPB = plane_items<R, NX, NY>();
-  constexpr int ML = kMaxLine<NX, NY>;
-  constexpr size_t smem = (size_t)IPB * NY * (NX + 1) * sizeof(cplx<R>);
-  if constexpr (sizeof(R) != 8) {
-    if (L.real_io) return false;
-  }
+  if (sizeof(R) != 8 && L.real_io) return false;
   if (L.prepare_only) {
-    if constexpr (!kSplitPlanes<R, NX, NY>) {   // whole lines per thread
-      if constexpr (sizeof(R) == 8) {
-        cudaFuncSetAttribute(pass_a_kernel<R, NX, NY, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(pass_a_kernel<R, NX, NY, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      }
-      cudaFuncSetAttribute(pass_a_kernel<R, NX, NY, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      cudaFuncSetAttribute(pass_c_kernel<R, NX, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      cudaFuncSetAttribute(pass_a_kernel<R, NX, NY, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      cudaFuncSetAttribute(pass_c_kernel<R, NX, NY>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    } else {
-      constexpr int s1 = (int)kSplitSmem<R, NX, NY>;
-      if constexpr (sizeof(R) == 8) {
-        cudaFuncSetAttribute(pass_a_split_kernel<R, NX, NY, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
-        cudaFuncSetAttribute(pass_a_split_kernel<R, NX, NY, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      }
-      cudaFuncSetAttribute(pass_a_split_kernel<R, NX, NY, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
-      cudaFuncSetAttribute(pass_c_split_kernel<R, NX, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
-      cudaFuncSetAttribute(pass_a_split_kernel<R, NX, NY, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      cudaFuncSetAttribute(pass_c_split_kernel<R, NX, NY>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    for (int q = 0; q <= 2; q += 2) {
+      launch_plane_as<R, NX, NY, false>(L, b, q, st);
+      launch_plane_as<R, NX, NY, true>(L, b, q, st);
     }
     return true;
   }
-  PlaneParams<R, NX, NY> P;
-  fill_plane<R, NX, NY>(P, L, b);
-  const long long items = (long long)b.npairs * L.nz;
-  const bool pdl = !L.no_pdl;
-  if constexpr (kSplitPlanes<R, NX, NY>) {
-    const dim3 grid((unsigned)items), blk(2 * ML);
-    if (pass == 0) {
-      if (sizeof(R) == 8 && L.real_io)
-        launch_pdl(pdl, pass_a_split_kernel<R, NX, NY, sizeof(R) == 8>, grid, blk, kSplitSmem<R, NX, NY>, st, P);
-      else
-        launch_pdl(pdl, pass_a_split_kernel<R, NX, NY, false>, grid, blk, kSplitSmem<R, NX, NY>, st, P);
-    } else {
-      launch_pdl(pdl, pass_c_split_kernel<R, NX, NY>, grid, blk, kSplitSmem<R, NX, NY>, st, P);
-    }
-  } else {
-    const dim3 grid((unsigned)((items + IPB - 1) / IPB)), blk(ML * IPB);
-    if (pass == 0) {
-      if (sizeof(R) == 8 && L.real_io)
-        launch_pdl(pdl, pass_a_kernel<R, NX, NY, sizeof(R) == 8>, grid, blk, smem, st, P);
-      else
-        launch_pdl(pdl, pass_a_kernel<R, NX, NY, false>, grid, blk, smem, st, P);
-    } else {
-      launch_pdl(pdl, pass_c_kernel<R, NX, NY>, grid, blk, smem, st, P);
-    }
-  }
+  if (L.V) launch_plane_as<R, NX, NY, true>(L, b, pass, st);
+  else launch_plane_as<R, NX, NY, false>(L, b, pass, st);
   return true;
 }
 
