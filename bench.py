@@ -109,7 +109,7 @@ def workload_config(name, s):
     return {"workload": name, "grid": f"{s.n}^3", "L_bohr": s.L, "n_occ": s.n_occ,
             "n_bands": s.n_bands, "kernel": f"erfc omega={s.omega}" if s.kernel == "erfc" else "bare",
             "orbitals": "seeded Gaussian-decaying plane waves |G|^2/2<=10 Ha, QR-orthonormal",
-            "precision": "fp32 pair/FFT path, TF32 3-term-split M and apply, fp64 Cholesky and L^-1, "
+            "precision": "fp32 pair/FFT path, TF32 3-term-split M, FP16-pair apply, fp64 Cholesky and L^-1, "
                          "Xi = W L^-* to fp64 accuracy (fp16 tensor-core slices)",
             "l2": "working set > L2 every step (no flush needed)"}
 
@@ -623,10 +623,10 @@ def xi_variants(ace, s, phi_d, reps, warm=True):
 
 
 def gemm_variants(ace, s, phi_d, psi_d, reps, warm=True):
-    """The dense products (M = dV Phi^* W, the apply) with the TF32 split (the
-    default) and the BF16 split (ACE_PREC_SPLIT_BF16): ms per ace_build and per
-    ace_apply with each, and the BF16 results' relative difference to the TF32
-    ones (M, V_ACE psi)."""
+    """The dense products (M = dV Phi^* W, the apply) by default ("tf32_split":
+    the TF32 split for M, FP16 pairs for an apply of this size) and with the BF16
+    split (ACE_PREC_SPLIT_BF16): ms per ace_build and per ace_apply with each, and
+    the BF16 results' relative difference to the default ones (M, V_ACE psi)."""
     import torch
     stream = torch.cuda.current_stream()
     out, res = {}, {}

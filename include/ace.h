@@ -77,13 +77,17 @@ typedef enum {
  * L^{-1} are FP64 in every mode.
  *  ACE_PREC_SPLIT_TF32: tcgen05 TF32 tensor cores for all three products, each
  *    FP32 operand split into two TF32 terms, three products (FP32 accuracy).
- *  ACE_PREC_XI_FP64 (the C64 default, ACE_PREC_DEFAULT): as SPLIT_TF32, except
- *    Xi = W L^{-*}, which is computed to FP64 accuracy from the FP32 W and the
+ *  ACE_PREC_XI_FP64 (the C64 default, ACE_PREC_DEFAULT): M as SPLIT_TF32. The
+ *    apply's products, from 2^16 grid points or 7 2^18 values in Xi and Psi together
+ *    on, run on the FP16 tensor cores: every vector scaled by a power of two, every value split into two
+ *    FP16 terms, three products (FP32 accuracy: an operand's error is below 2^-22 of
+ *    itself, or 2^-40 of its vector's largest value if that is more); smaller
+ *    calls as SPLIT_TF32. Xi = W L^{-*} is computed to FP64 accuracy from the FP32 W and the
  *    FP64 L^{-*} on the FP16 tensor cores (error-free 8-bit integer slices of
  *    both operands, exact integer products, exact accumulation) and rounded
  *    once to FP32: before that rounding the error of Xi_b(g) is below about
  *    2^-41 max_k |W_k(g)| sum_k |(L^{-*})_kb|.
- *  ACE_PREC_XI_FP64_SIMT: the same Xi with plain FP64 arithmetic on CUDA cores.
+ *  ACE_PREC_XI_FP64_SIMT: the same, with Xi by plain FP64 arithmetic on CUDA cores.
  *  ACE_PREC_FP32: all three products in FP32 on CUDA cores.
  *  ACE_PREC_SPLIT_BF16: M = dV Phi^* W and the apply's two products on tcgen05
  *    BF16 tensor cores, each FP32 operand split into two BF16 terms (hi = the
@@ -347,7 +351,7 @@ ace_status ace_profile_end(ace_plan* plan, double* ms_out, long long* counts_out
  * the GPU (other streams, other plans) race and must be serialised by the
  * caller. Nothing needs clearing between calls. The GEMMs run on CUDA cores:
  * for FP64 plans the result equals ace_apply's up to the order of the split-K
- * sums; for ACE_DTYPE_C64 plans, whose ace_apply uses the TF32 3-term-split
+ * sums; for ACE_DTYPE_C64 plans, whose ace_apply uses split operands on the
  * tensor cores, the two agree to the FP32 apply tolerance (about 1e-6
  * relative), not bit for bit. Calls no allocator. */
 ace_status ace_apply_static(ace_plan* plan, const void* Xi, const void* Psi, int n_b, void* Y,

@@ -20,7 +20,7 @@ LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libace.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
-PLAIN = ["pair_dispatch.cu", "pair_point.cu", "dense.cu", "chol.cu", "tc_gemm.cu", "xi_oz.cu", "ace_api.cu",
+PLAIN = ["pair_dispatch.cu", "pair_point.cu", "dense.cu", "chol.cu", "tc_gemm.cu", "tc_apply.cu", "xi_oz.cu", "ace_api.cu",
          "apply_static.cu"]
 
 

@@ -102,6 +102,7 @@ struct ace_plan {
   bool graphs = true;
   bool engine = true;            // persistent pair engine (else four kernels per batch)
   bool tc = false;               // tensor-core GEMMs (complex FP32 storage)
+  bool apply16 = false;          // the apply with FP16 operand pairs (tc_apply.cu)
   bool bf16 = false;             // M and the apply with BF16 operands (ACE_PREC_SPLIT_BF16)
   bool overlap = false;          // graph mode: one chain of passes (FP32), or pass A of batch k+1 beside pass D of batch k (FP64)
   int radix = 0;                 // line-transform radix order (ACE_FLAG_RADIX_ODD_FIRST)
@@ -350,6 +351,7 @@ WsLayout layout(const ace_plan* p, int op, int nb, char* base) {
   if (op == ACE_OP_APPLY) {
     L.part = (double*)take((size_t)splits * N * nb * 2 * sizeof(double));
     L.Cm = (double*)take((size_t)N * nb * 2 * sizeof(double));
+    if (p->apply16 && nb > 0 && off < apply_tc_scratch_bytes(p->ng, N, nb)) off = apply_tc_scratch_bytes(p->ng, N, nb);
   }
   L.total = off;
   return L;
@@ -850,6 +852,7 @@ ace_status ace_plan_create(const ace_desc* d, ace_plan** out) {
   // C64 default: Xi to FP64 accuracy on the FP16 tensor cores (the triangular
   // product stays FP64-accurate, as the Cholesky factor it applies)
   p->bf16 = p->tc && d->prec == ACE_PREC_SPLIT_BF16;
+  p->apply16 = p->tc && !p->bf16 && d->prec != ACE_PREC_SPLIT_TF32;
   const bool xi_slices = d->prec == ACE_PREC_XI_FP64 || d->prec == ACE_PREC_SPLIT_BF16 ||
                          (d->prec == ACE_PREC_DEFAULT && p->tc);
   p->xi = xi_slices ? 1 : (d->prec == ACE_PREC_XI_FP64_SIMT ? 2 : 0);
@@ -944,6 +947,7 @@ ace_status ace_plan_create(const ace_desc* d, ace_plan** out) {
     launch_one(p, prep, none, nullptr);
     prepare_cholesky(N);
     if (p->tc) tc_gemm_prepare();
+    if (p->apply16) apply_tc_prepare();
     if (p->xi == 1) xi_oz_prepare();
     if (p->engine) {
       if (p->f64) engine_prepare_f64(p->nx, p->einfo);
@@ -1416,8 +1420,14 @@ ace_status ace_apply(ace_plan* p, const void* Xi, const void* Psi, int nb, void*
   cudaStream_t st = (cudaStream_t)stream;
   const int N = p->d.n_occ;
   const WsLayout Wl = layout(p, ACE_OP_APPLY, nb, (char*)ws);
-  const int splits = gram_parts(p, N, nb);
   // C = dV Xi^* Psi, Y = -Xi C (Eq. ACE)
+  if (p->apply16 && apply_tc_faster(p->ng, N, nb)) {
+    const int k = launch_apply_tc(Xi, N, Psi, nb, p->ld, p->ng, p->dv, Y, ws, p->status, st);
+    if (k == 0) return fail(ACE_ERR_CUDA, "tensor map encoding failed");
+    p->launches += k;
+    return cuda_check("ace_apply");
+  }
+  const int splits = gram_parts(p, N, nb);
   if (p->tc) launch_gram_tc(Xi, N, Psi, nb, p->ld, p->ng, Wl.part, splits, p->status, st, p->bf16);
   else launch_gram(p->f64, p->real, Xi, N, Psi, nb, p->ld, p->ng, Wl.part, splits, st);
   launch_gram_reduce(Wl.part, splits, N, nb, p->dv, false, false, Wl.Cm, nullptr, st);
