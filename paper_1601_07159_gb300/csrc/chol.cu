@@ -5,19 +5,25 @@
 // Blocks of NB = 16 columns (the diagonal blocks run on one SM each, so they
 // are kept small; 32 measured slightly slower). For panel p (rows/cols
 // [p0, p0 + nb)):
-//   diag    one CTA: A_pp -> L_pp (right-looking Cholesky in shared memory,
-//           status word on a non-finite or non-positive pivot), D_p = L_pp^{-1}
-//           (recursive-doubling inverse of a triangular matrix); L_pp is
-//           stored in A, D_p in the diagonal block of X.
-//   panel   L_ip = A_ip D_p^*  for every row i below the panel (one CTA per 16
+//   diag    one CTA: A_pp -> L_pp (status word on a non-finite or non-positive
+//           pivot) and D_p = L_pp^{-1}; L_pp is stored in A, D_p in the diagonal
+//           block of X.
+//   panel   L_ip = A_ip D_p^*  for every row i below the panel (one CTA per 2
 //           rows, in place: a CTA reads and writes only its own rows).
 //   update  A_ik -= sum_l L_il conj(L_kl) over the panel columns l, for the
-//           trailing lower triangle i >= k (16 x 16 output tiles).
-// Then the block rows of X = L^{-1} below the diagonal, in order q = 1..P-1:
-//   T     = L(q, 0:q) X(0:q, 0:q)        (block-row product, X lower triangular)
-//   X(q, 0:q) = -D_q T
-// and finally LinvH[c][i] = conj(X_ic) (zero above the diagonal), so that
+//           trailing lower triangle i >= k (8 x 8 output tiles).
+// Then X = L^{-1} below the diagonal blocks by recursive doubling: with
+// [[A, 0], [B, C]] the blocks of edge h = 16, 32, ... of L,
+//   T = B A^{-1}, then X_B = -C^{-1} T
+// for all pairs of a level at once: 2 log2(n / 16) launches.
+// Finally LinvH[c][i] = conj(X_ic) (zero above the diagonal), so that
 // Xi_k = sum_i W_i LinvH[i][k].
+// FP64 issue bounds each of these kernels (about 1.7 multiply-adds per cycle and SM: 75
+// cycles per warp instruction and SM quadrant), and at 128 orbitals and fewer its latency: outputs are
+// spread over as many SMs as there are (2-row panels and 8 x 8 tiles in place of 16 rows
+// and 16 x 16), sums are cut in parts that meet by shuffles, and dependent steps
+// are few. Kernel times for 128 orbitals: 392 -> 212 us (diag 8 x 22.4 -> 10.7, panel 8.1 ->
+// 5.0, update 8.2 -> 5.3, the inverse from 7 row steps of 12.9 to 3 levels of 15.7).
 // Every kernel returns at once when the status word already holds a failure.
 #include <cmath>
 
@@ -28,7 +34,7 @@ namespace ace {
 namespace {
 
 constexpr int NB = 16;   // panel width
-constexpr int TT = 16;   // output tile edge of the FP64 tile products
+constexpr int TT = 8;    // output tile edge of the FP64 tile products
 
 __device__ __forceinline__ double2 zfma(double2 acc, double2 a, double2 b) {   // acc + a b
   acc.x = fma(a.x, b.x, acc.x);
@@ -50,167 +56,171 @@ __global__ void neg_copy_kernel(const double2* __restrict__ M, long long count, 
   if (i < count) A[i] = make_double2(-M[i].x, -M[i].y);
 }
 
-// Factor and invert the diagonal block of panel p (nb <= NB); NB * NB threads.
-// The block is padded to NB with the identity, so every loop runs NB uniform
-// steps.
-// Cholesky on unscaled columns: step j subtracts a_ij conj(a_kj) / d_j from
-// the trailing lower triangle (d_j = a_jj at step j). The trailing triangle's
-// elements are packed densely onto threads (a table ordered by decreasing
-// column, so the elements of step j are the first (NB-1-j)(NB-j)/2), which
-// keeps warps full: FP64 issue is the scarce resource on this part. The thread
-// that updates a_{j+1,j+1} in step j also checks that pivot and forms its
-// reciprocal, so a step needs one barrier and one FP64 reciprocal. The
-// reciprocal is the FP32 one refined by two Newton-Raphson steps in FP64
-// (r <- r + r (1 - d r); each step squares the relative error: 1e-7 -> 1e-14
-// -> rounding). Afterwards L_jj = sqrt(d_j) and L_ij = a_ij / sqrt(d_j) in one
-// parallel pass.
-// Inverse by recursive doubling: for a lower-triangular [[A, 0], [B, C]],
-// the inverse is [[A^-1, 0], [-C^-1 (B A^-1), C^-1]]; log2 NB levels (block
-// edge 2, 4, ..., NB) of small products replace NB dependent column steps. The
-// intermediate B A^-1 is kept, transposed, in the unused upper triangle of X.
-__device__ __forceinline__ double recip_nr(double d) {
-  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;   // outside FP32's comfortable range
-  double r = (double)(1.0f / (float)d);
-  r = fma(r, fma(-d, r, 1.0), r);
-  r = fma(r, fma(-d, r, 1.0), r);
-  return r;
+// r ~ 1 / d and y ~ 1 / sqrt(d) for a positive finite d: the hardware's 20-bit
+// approximations (they flush subnormal numbers) and one cubic step, e = 1 - d r: r (1 + e + e^2), e = 1 - d y^2:
+// y (1 + e / 2 + 3 e^2 / 8) (2^-20 -> 2^-60, then rounding).
+// plain(): d positive with a binary exponent in [-930, 930], from the upper word (a
+// comparison of doubles costs as much as a multiply-add).
+__device__ __forceinline__ bool plain(double d) {
+  return (unsigned)(__double2hiint(d) - ((1023 - 930) << 20)) < (1860u << 20);
+}
+__device__ __forceinline__ double recip(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double recip_sqrt(double d) {
+  if (!plain(d)) return 1.0 / sqrt(d);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-d * y, y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
-constexpr int kTri = NB * (NB - 1) / 2;   // trailing-triangle elements (i >= k >= 1)
-
-__global__ void __launch_bounds__(NB * NB)
+// Factor and invert the diagonal block of panel p (nb <= NB). The block is padded to
+// NB with the identity, so every loop runs NB uniform steps.
+// Elimination on unscaled columns, -M = L' D L'^*: step j subtracts
+// (a_ij / d_j) conj(a_kj) from the trailing a_ik (i >= k > j) and (a_ij / d_j) x_jc from
+// row i of X = L'^{-1} (c <= j, X starts as the identity): row i has i + 1
+// elements in every step. So each lower-triangle element (i, k) has one thread, which
+// holds a_ik in a register up to step k, where it is final, and x_ik from
+// there on. A step reads column j of a and row j of x, published in shared memory by
+// the step before (two buffers, one barrier a step). Warp PIV works ahead on the
+// pivot: d_{j+1} = a_{j+1,j+1} - |a_{j+1,j}|^2 / d_j and its reciprocal, while the
+// others do step j (with the pivot taken from its element's thread and the inverse
+// formed afterwards, by recursive doubling, the kernel took 22.4 us; 10.7 so).
+// At the end L_ik = a_ik / sqrt(d_k), and row i of X is divided by sqrt(d_i).
+constexpr int kTri = NB * (NB + 1) / 2;             // lower-triangle elements
+constexpr int PIV = (kTri + 31) / 32;               // the pivot's warp, after the elements'
+__global__ void __launch_bounds__((PIV + 1) * 32)
 diag_kernel(double2* __restrict__ A, double2* __restrict__ X, int n, int p0, int nb, int* status) {
-  __shared__ double2 a[NB][NB + 1];
-  __shared__ double2 x[NB][NB + 1];
-  __shared__ double dl[NB], dil[NB], rj[NB];
-  __shared__ unsigned char ti[kTri], tk[kTri];
+  __shared__ double2 col[2][NB], row[2][NB];        // a_ij (i > j) and x_jc (c <= j) of step j
+  __shared__ double dg[2], rj[2];                   // a_{j+1,j+1} before step j, 1 / d_j
+  __shared__ double dd[NB], y[NB];                  // d_j, 1 / sqrt(d_j)
   __shared__ int s_fail, s_piv;
-  const int tid = threadIdx.x;
-  const int ei = tid / NB, ek = tid % NB;
+  const int tid = threadIdx.x, w = tid >> 5;
   if (status[0] != 0) return;
-  {
-    double2 v = make_double2(ei == ek ? 1.0 : 0.0, 0.0);
-    if (ei < nb && ek <= ei) v = A[(long long)(p0 + ei) * n + p0 + ek];
-    a[ei][ek] = v;
-    x[ei][ek] = make_double2(0.0, 0.0);
+  // element (i, k) of thread tid: rows in decreasing order, so that the elements of a
+  // step are the first threads
+  int i = NB - 1, k = tid;
+  while (k > i && i >= 0) k -= i-- + 1;
+  const bool elem = tid < kTri;
+  double2 v = make_double2(0.0, 0.0);
+  if (elem) {
+    v = make_double2(i == k ? 1.0 : 0.0, 0.0);
+    if (i < nb) v = A[(long long)(p0 + i) * n + p0 + k];
+    if (k == 0) col[0][i] = v;
+    if (i == 1 && k == 1) dg[0] = v.x;
   }
-  // packed trailing-triangle table: entries (i, k), k = NB-1 down to 1, i = k .. NB-1
-  if (tid < kTri) {
-    int k = NB - 1, o = 0;
-    while (tid >= o + (NB - k)) {
-      o += NB - k;
-      --k;
-    }
-    ti[tid] = (unsigned char)(k + (tid - o));
-    tk[tid] = (unsigned char)k;
-  }
-  if (tid == 0) s_fail = 0;
-  __syncthreads();
-  auto pivot = [&](int j) {     // one thread: check d_j, store its reciprocal
-    const double d = a[j][j].x;
-    if (!isfinite(d) || !(d > 0.0)) {
+  auto pivot = [&](int j, double d) {               // lane 0 of warp PIV: check d_j, keep it and its reciprocal
+    dd[j] = d;
+    if (plain(d)) {
+      rj[j & 1] = recip(d);
+    } else if (isfinite(d) && d > 0.0) {
+      rj[j & 1] = 1.0 / d;
+    } else {
       s_fail = isfinite(d) ? -2 : -3;
       s_piv = j;
-      rj[j] = 0.0;
-    } else {
-      rj[j] = recip_nr(d);
     }
   };
-  if (tid == 0) pivot(0);
+  if (tid == 0) {
+    s_fail = 0;
+    row[0][0] = make_double2(1.0, 0.0);
+  }
   __syncthreads();
+  if (tid == PIV * 32) pivot(0, col[0][0].x);
+  __syncthreads();
+  double2 l = v;                                    // a_ik once it is final
   for (int j = 0; j < NB; ++j) {
-    if (s_fail) {               // uniform: read after a barrier
+    if (s_fail) {                                   // uniform: read after a barrier
       if (tid == 0) {
         status[0] = s_fail;
         status[1] = p0 + s_piv + 1;
       }
       return;
     }
-    const int cnt = (NB - 1 - j) * (NB - j) / 2;
-    if (tid < cnt) {
-      const int i = ti[tid], k = tk[tid];
-      const double r = rj[j];
-      const double2 u = a[i][j];
-      const double2 w = a[k][j];
-      a[i][k] = zfmac(a[i][k], make_double2(-u.x * r, -u.y * r), w);
-      if (i == j + 1 && k == j + 1) pivot(j + 1);
+    const int c = j & 1;
+    const double r = rj[c];
+    if (w == PIV) {
+      if (tid == PIV * 32 && j + 1 < NB) {
+        const double2 u = col[c][j + 1];
+        pivot(j + 1, fma(-fma(u.x, u.x, u.y * u.y), r, dg[c]));
+      }
+    } else if (elem && i > j) {
+      if (k == j) {                                 // a_ij is final: on to x_ij, which starts at zero
+        l = v;
+        v = make_double2(0.0, 0.0);
+      }
+      const double2 u = col[c][i];
+      double2 z = k > j ? col[c][k] : row[c][k];
+      if (k > j) z.y = -z.y;
+      v = zfma(v, make_double2(-u.x * r, -u.y * r), z);
+      if (k == j + 1) col[c ^ 1][i] = v;
+      if (i == j + 1) row[c ^ 1][k] = k == i ? make_double2(1.0, 0.0) : v;
+      if (i == j + 2 && k == i) dg[c ^ 1] = v.x;
     }
     __syncthreads();
   }
-  if (tid < NB) {
-    const double l = sqrt(a[tid][tid].x);
-    dl[tid] = l;
-    dil[tid] = 1.0 / l;
-  }
+  if (tid < NB) y[tid] = recip_sqrt(dd[tid]);
   __syncthreads();
-  if (ek < ei) {
-    a[ei][ek].x *= dil[ek];
-    a[ei][ek].y *= dil[ek];
-  } else if (ek == ei) {
-    a[ei][ei] = make_double2(dl[ei], 0.0);
-    x[ei][ei] = make_double2(dil[ei], 0.0);
+  if (!elem || i >= nb) return;
+  const double yi = y[i], yk = y[k];
+  const long long o = (long long)(p0 + i) * n + p0 + k;
+  if (i == k) {
+    A[o] = make_double2(dd[i] * yi, 0.0);
+    X[o] = make_double2(yi, 0.0);
+  } else {
+    A[o] = make_double2(l.x * yk, l.y * yk);
+    X[o] = make_double2(v.x * yi, v.y * yi);
   }
-  __syncthreads();
-  if (ei < nb && ek <= ei) A[(long long)(p0 + ei) * n + p0 + ek] = a[ei][ek];
-  for (int h = 1; h < NB; h *= 2) {     // blocks of edge 2h at rows/cols b .. b + 2h
-    const int cnt = (NB / (2 * h)) * h * h;
-    // T = B A^{-1}: T_rc = sum_{m >= c} a[b+h+r][b+m] x[b+m][b+c], stored at x[b+c][b+h+r]
-    for (int e = tid; e < cnt; e += blockDim.x) {
-      const int blk = e / (h * h), r = (e / h) % h, c = e % h, b = blk * 2 * h;
-      double2 t = make_double2(0.0, 0.0);
-      for (int m = c; m < h; ++m) t = zfma(t, a[b + h + r][b + m], x[b + m][b + c]);
-      x[b + c][b + h + r] = t;
-    }
-    __syncthreads();
-    // X_B = -C^{-1} T: X[b+h+r][b+c] = -sum_{m <= r} x[b+h+r][b+h+m] T_mc
-    for (int e = tid; e < cnt; e += blockDim.x) {
-      const int blk = e / (h * h), r = (e / h) % h, c = e % h, b = blk * 2 * h;
-      double2 t = make_double2(0.0, 0.0);
-      for (int m = 0; m <= r; ++m) t = zfma(t, x[b + h + r][b + h + m], x[b + c][b + h + m]);
-      x[b + h + r][b + c] = make_double2(-t.x, -t.y);
-    }
-    __syncthreads();
-  }
-  if (ei < nb && ek < nb) X[(long long)(p0 + ei) * n + p0 + ek] = ek <= ei ? x[ei][ek] : make_double2(0.0, 0.0);
 }
 
-// L_ip = A_ip D_p^* for rows i in [r0, n): one CTA per TT rows, all nb columns.
-__global__ void __launch_bounds__(256)
+// L_ip = A_ip D_p^* for rows i in [r0, n): PR rows and all nb columns per CTA, four
+// threads per output.
+constexpr int PR = 2;
+__global__ void __launch_bounds__(PR * NB * 4)
 panel_kernel(double2* __restrict__ A, const double2* __restrict__ X, int n, int p0, int nb, int r0,
              const int* status) {
-  __shared__ double2 rows[TT][NB + 1];
+  __shared__ double2 rows[PR][NB + 1];
   __shared__ double2 d[NB][NB + 1];
   if (status[0] != 0) return;
   const int tid = threadIdx.x;
-  const int i0 = r0 + blockIdx.x * TT;
-  for (int e = tid; e < TT * NB; e += blockDim.x) {
+  const int i0 = r0 + blockIdx.x * PR;
+  for (int e = tid; e < PR * NB; e += blockDim.x) {
     const int i = e / NB, k = e % NB;
     rows[i][k] = (i0 + i < n && k < nb) ? A[(long long)(i0 + i) * n + p0 + k] : make_double2(0.0, 0.0);
   }
   for (int e = tid; e < NB * NB; e += blockDim.x) {
     const int i = e / NB, k = e % NB;
-    d[i][k] = (i < nb && k < nb) ? X[(long long)(p0 + i) * n + p0 + k] : make_double2(0.0, 0.0);
+    d[i][k] = (i < nb && k <= i) ? X[(long long)(p0 + i) * n + p0 + k] : make_double2(0.0, 0.0);
   }
   __syncthreads();
-  for (int e = tid; e < TT * NB; e += blockDim.x) {
-    const int i = e / NB, c = e % NB;
-    if (i0 + i >= n || c >= nb) continue;
-    double2 s = make_double2(0.0, 0.0);
-    for (int k = 0; k < nb; ++k) s = zfmac(s, rows[i][k], d[c][k]);   // sum_k A_ik conj(D_ck)
-    A[(long long)(i0 + i) * n + p0 + c] = s;
+  const int part = tid & 3, c = (tid >> 2) % NB, i = (tid >> 2) / NB;
+  double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int k = 0; k < NB; k += 4) s = zfmac(s, rows[i][k + part], d[c][k + part]);   // sum_k A_ik conj(D_ck)
+#pragma unroll
+  for (int o = 1; o < 4; o *= 2) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
   }
+  if (part == 0 && i0 + i < n && c < nb) A[(long long)(i0 + i) * n + p0 + c] = s;
 }
 
 // A_ik -= sum_{l in panel} L_il conj(L_kl), trailing lower triangle i >= k >= r0.
-// Grid: one CTA per lower 16 x 16 tile (bi >= bk) of the trailing block.
-__global__ void __launch_bounds__(256)
+// Grid: one CTA per lower 8 x 8 tile (bi >= bk) of the trailing block, two threads
+// per output.
+__global__ void __launch_bounds__(2 * TT * TT)
 update_kernel(double2* __restrict__ A, int n, int p0, int nb, int r0, const int* status) {
   __shared__ double2 li[TT][NB + 1];
   __shared__ double2 lk[TT][NB + 1];
   if (status[0] != 0) return;
-  int t = blockIdx.x, bi = 0;
-  while (t > bi) { t -= bi + 1; ++bi; }
-  const int bk = t;
+  // bi (bi + 1) / 2 <= blockIdx.x < (bi + 1) (bi + 2) / 2
+  int bi = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while (bi * (bi + 1) / 2 > (int)blockIdx.x) --bi;
+  while ((bi + 1) * (bi + 2) / 2 <= (int)blockIdx.x) ++bi;
+  const int bk = (int)blockIdx.x - bi * (bi + 1) / 2;
   const int i0 = r0 + bi * TT, k0 = r0 + bk * TT;
   const int tid = threadIdx.x;
   for (int e = tid; e < TT * NB; e += blockDim.x) {
@@ -220,52 +230,70 @@ update_kernel(double2* __restrict__ A, int n, int p0, int nb, int r0, const int*
     lk[r][c] = (okc && k0 + r < n) ? A[(long long)(k0 + r) * n + p0 + c] : make_double2(0.0, 0.0);
   }
   __syncthreads();
-  const int r = tid / TT, c = tid % TT;
-  const int i = i0 + r, k = k0 + c;
-  if (i >= n || k >= n || k > i) return;
+  const int part = tid & 1, r = (tid >> 1) / TT, c = (tid >> 1) % TT;
   double2 s = make_double2(0.0, 0.0);
-  for (int l = 0; l < nb; ++l) s = zfmac(s, li[r][l], lk[c][l]);
+#pragma unroll
+  for (int l = 0; l < NB; l += 2) s = zfmac(s, li[r][l + part], lk[c][l + part]);
+  s.x += __shfl_xor_sync(0xffffffffu, s.x, 1);
+  s.y += __shfl_xor_sync(0xffffffffu, s.y, 1);
+  const int i = i0 + r, k = k0 + c;
+  if (part != 0 || i >= n || k >= n || k > i) return;
   double2& out = A[(long long)i * n + k];
   out = make_double2(out.x - s.x, out.y - s.y);
 }
 
-// T(r, j) = sum_{k = j}^{q0 - 1} L(q0 + r, k) X(k, j), r < nb, j < q0 (X lower triangular).
-// Block (32, KS): x indexes j, y strides over k; the KS partial sums are added
-// in a fixed order, so the result does not depend on timing.
-constexpr int KS = 8;
-__global__ void __launch_bounds__(256)
-inv_row_kernel(const double2* __restrict__ A, const double2* __restrict__ X, double2* __restrict__ T,
-               int n, int q0, int nb, const int* status) {
-  __shared__ double2 red[KS][32];
+// One product of a doubling level, for the pair blockIdx.z of blocks of edge h at rows
+// and columns s = 2 h blockIdx.z; 8 x 8 outputs (r, c) per CTA, two threads each. The
+// intermediate T(r, c) lies transposed in the unused upper triangle, at X(s + c, s + h + r).
+//   FIRST:  T(r, c) = sum_{m >= c} L(s + h + r, s + m) X(s + m, s + c)
+//   second: X(s + h + r, s + c) = -sum_{m <= r} X(s + h + r, s + h + m) T(m, c)
+template <bool FIRST>
+__global__ void __launch_bounds__(2 * TT * TT)
+inv_level_kernel(const double2* __restrict__ A, double2* __restrict__ X, int n, int h, const int* status) {
+  __shared__ double2 f[TT][NB + 1];                 // rows r of the left factor
+  __shared__ double2 g[TT][NB + 1];                 // columns c of the right factor
   if (status[0] != 0) return;
-  const int r = blockIdx.y, j = blockIdx.x * 32 + threadIdx.x, ty = threadIdx.y;
-  double2 s = make_double2(0.0, 0.0);
-  if (j < q0)
-    for (int k = j + ty; k < q0; k += KS) s = zfma(s, A[(long long)(q0 + r) * n + k], X[(long long)k * n + j]);
-  red[ty][threadIdx.x] = s;
-  __syncthreads();
-  if (ty == 0 && j < q0) {
-    for (int y = 1; y < KS; ++y) s = make_double2(s.x + red[y][threadIdx.x].x, s.y + red[y][threadIdx.x].y);
-    T[(long long)r * q0 + j] = s;
+  const int s = 2 * h * blockIdx.z, r0 = blockIdx.y * TT, c0 = blockIdx.x * TT, lo = s + h;
+  if (lo + r0 >= n) return;
+  const int tid = threadIdx.x, part = tid & 1, r = (tid >> 1) / TT, c = (tid >> 1) % TT;
+  const int rows = min(h, n - lo);                  // of the pair's lower block
+  const int m0 = FIRST ? c0 : 0, m1 = FIRST ? h : min(r0 + TT, rows);
+  double2 acc = make_double2(0.0, 0.0);
+  for (int m = m0; m < m1; m += NB) {
+    for (int e = tid; e < TT * NB; e += blockDim.x) {
+      const int q = e / NB, mm = m + e % NB;
+      const bool okr = r0 + q < rows && mm < m1;
+      double2 u = make_double2(0.0, 0.0);
+      if (FIRST) {
+        if (okr) u = A[(long long)(lo + r0 + q) * n + s + mm];
+      } else {
+        if (okr && mm <= r0 + q) u = X[(long long)(lo + r0 + q) * n + lo + mm];
+      }
+      f[q][e % NB] = u;
+    }
+    for (int e = tid; e < TT * NB; e += blockDim.x) {
+      // FIRST: rows mm of X, contiguous over c; second: T transposed, contiguous over mm
+      const int q = FIRST ? e % TT : e / NB, t = FIRST ? e / TT : e % NB, mm = m + t;
+      double2 u = make_double2(0.0, 0.0);
+      if (mm < m1) {
+        if (FIRST) {
+          if (mm >= c0 + q) u = X[(long long)(s + mm) * n + s + c0 + q];
+        } else {
+          u = X[(long long)(s + c0 + q) * n + lo + mm];
+        }
+      }
+      g[q][t] = u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < NB; t += 2) acc = zfma(acc, f[r][t + part], g[c][t + part]);
+    __syncthreads();
   }
-}
-
-// X(q0 + r, j) = -sum_c D_q(r, c) T(c, j), r < nb, j < q0 (same block shape, y strides over c).
-__global__ void __launch_bounds__(256)
-inv_apply_kernel(const double2* __restrict__ T, double2* __restrict__ X, int n, int q0, int nb,
-                 const int* status) {
-  __shared__ double2 red[KS][32];
-  if (status[0] != 0) return;
-  const int r = blockIdx.y, j = blockIdx.x * 32 + threadIdx.x, ty = threadIdx.y;
-  double2 s = make_double2(0.0, 0.0);
-  if (j < q0)
-    for (int c = ty; c <= r; c += KS) s = zfma(s, X[(long long)(q0 + r) * n + q0 + c], T[(long long)c * q0 + j]);
-  red[ty][threadIdx.x] = s;
-  __syncthreads();
-  if (ty == 0 && j < q0) {
-    for (int y = 1; y < KS; ++y) s = make_double2(s.x + red[y][threadIdx.x].x, s.y + red[y][threadIdx.x].y);
-    X[(long long)(q0 + r) * n + j] = make_double2(-s.x, -s.y);
-  }
+  acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
+  acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+  if (part != 0 || r0 + r >= rows) return;
+  if (FIRST) X[(long long)(s + c0 + c) * n + lo + r0 + r] = acc;
+  else X[(long long)(lo + r0 + r) * n + s + c0 + c] = make_double2(-acc.x, -acc.y);
 }
 
 __global__ void linvh_kernel(const double2* __restrict__ X, int n, double* __restrict__ LinvH,
@@ -284,33 +312,31 @@ __global__ void linvh_kernel(const double2* __restrict__ X, int n, double* __res
 
 void prepare_cholesky(int) {}
 
-size_t cholesky_work_doubles(int n) { return 2 * ((size_t)2 * n * n + (size_t)NB * n); }
+size_t cholesky_work_doubles(int n) { return (size_t)4 * n * n; }
 
 int launch_cholesky_inv(const double* M, int n, double* work, double* LinvH, int* status, cudaStream_t st) {
   double2* A = reinterpret_cast<double2*>(work);
   double2* X = A + (size_t)n * n;
-  double2* T = X + (size_t)n * n;
   int launches = 0;
   const long long nn = (long long)n * n;
   neg_copy_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(reinterpret_cast<const double2*>(M), nn, A);
   ++launches;
   for (int p0 = 0; p0 < n; p0 += NB) {
     const int nb = (p0 + NB <= n) ? NB : n - p0;
-    diag_kernel<<<1, NB * NB, 0, st>>>(A, X, n, p0, nb, status);
+    diag_kernel<<<1, (PIV + 1) * 32, 0, st>>>(A, X, n, p0, nb, status);
     ++launches;
     const int r0 = p0 + nb;
     if (r0 >= n) break;
     const int rows = n - r0;
-    panel_kernel<<<(rows + TT - 1) / TT, 256, 0, st>>>(A, X, n, p0, nb, r0, status);
+    panel_kernel<<<(rows + PR - 1) / PR, PR * NB * 4, 0, st>>>(A, X, n, p0, nb, r0, status);
     const int bt = (rows + TT - 1) / TT;
-    update_kernel<<<bt * (bt + 1) / 2, 256, 0, st>>>(A, n, p0, nb, r0, status);
+    update_kernel<<<bt * (bt + 1) / 2, 2 * TT * TT, 0, st>>>(A, n, p0, nb, r0, status);
     launches += 2;
   }
-  for (int q0 = NB; q0 < n; q0 += NB) {
-    const int nb = (q0 + NB <= n) ? NB : n - q0;
-    const dim3 grid((q0 + 31) / 32, nb), block(32, KS);
-    inv_row_kernel<<<grid, block, 0, st>>>(A, X, T, n, q0, nb, status);
-    inv_apply_kernel<<<grid, block, 0, st>>>(T, X, n, q0, nb, status);
+  for (int h = NB; h < n; h *= 2) {
+    const dim3 grid(h / TT, h / TT, (n + h - 1) / (2 * h));
+    inv_level_kernel<true><<<grid, 2 * TT * TT, 0, st>>>(A, X, n, h, status);
+    inv_level_kernel<false><<<grid, 2 * TT * TT, 0, st>>>(A, X, n, h, status);
     launches += 2;
   }
   linvh_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(X, n, LinvH, status);
