@@ -33,15 +33,19 @@
 //   and scaled by the power of two (exact), in FP32 for FP32 outputs (no FP64
 //   arithmetic, which is slow on this part).
 //
-// Per CTA (512 threads, one per SM): T - 1 accumulators of TN columns in TMEM;
-// K runs in chunks of 32 real terms (16 orbitals) through three shared-memory
-// stages, each holding T - 1 A slices (split on the fly from the FP32 loads) and
-// the chunk's B slices (split once per call by oz_slice_b_kernel into the
-// stage layout, brought in by one bulk copy per chunk on the TMA unit, which
-// completes on the stage's second mbarrier). One thread issues the bulk copy
-// and, once it has landed, the MMAs of the chunk (2 K-steps per slice pair),
-// and commits them to the stage's first mbarrier;
-// the threads drain the accumulators after the last chunk of each group.
+// Per CTA (16 working warps and one that issues, one CTA per SM): T - 1 accumulators of TN
+// columns in TMEM; K runs in chunks of 32 real terms (16 orbitals) through three
+// shared-memory stages, each holding T - 1 A slices (split on the fly from the FP32
+// loads) and the chunk's B slices (split once per call by oz_slice_b_kernel into the
+// stage layout). The CTA's tiles are one stream of chunks. One thread of the
+// issuing warp brings the B slices of the next chunk by a bulk copy, waits for a chunk's A
+// and B slices, issues its MMAs (2 K-steps per slice pair) and commits them. The
+// working warps run up to two chunks ahead, each waiting for no more than the MMAs that
+// last read its stage, and read a group's accumulators back after storing the
+// chunk that follows it. They meet the issuing warp on mbarriers alone: with one
+// thread of the sixteen warps issuing copy and MMAs between two block-wide barriers a
+// chunk, every chunk waited for its own copy and for the 30 MMAs to be issued
+// (128 orbitals of 48^3: 516 us; 359 us so).
 // L^{-*} is upper triangular, so tile [b0, b0 + BB) runs k < b0 + BB only.
 // Every mbarrier wait is bounded: on timeout the CTA records ACE_ERR_TIMEOUT,
 // stops issuing, waits (bounded) for what it issued and frees its TMEM.
@@ -55,7 +59,12 @@ namespace ace {
 
 namespace {
 
-constexpr int OZ_THREADS = 512;
+constexpr int OZ_WORKERS = 512;                // threads that split A and read the accumulators
+constexpr int OZ_THREADS = OZ_WORKERS + 128;   // and the issuing warp's group (registers move by groups of four warps)
+// registers a thread: 96 at launch (five warps per SM quadrant); the issuing group keeps 24
+// and the workers take 112: 512 x 112 + 128 x 24 = 60416 of the launch's 640 x 96 = 61440
+constexpr int OZ_REG_ISSUE = 24, OZ_REG_WORK = 112;
+static_assert(OZ_WORKERS * OZ_REG_WORK + 128 * OZ_REG_ISSUE <= OZ_THREADS * 96, "register split");
 constexpr int OZ_TM = 128;                     // rows per CTA (M of the MMA)
 constexpr int OZ_KC = 32;                      // real K terms per chunk
 constexpr int OZ_SBO = (OZ_KC / 8) * 128;      // bytes between 8-row groups of 16-bit elements = 512
@@ -68,14 +77,13 @@ template <int T> struct Oz {
   static_assert(T == 5 || T == 6, "slice depth");
   static constexpr int SA = T - 1;             // A slices: 8 (T - 1) bits below the row maximum
   static constexpr int SB = T - 1;             // C slices
-  static constexpr int NW = T - 1;             // accumulators, weights w = 2 .. T
-  static constexpr int TN = T == 5 ? 128 : 96; // NW x TN <= 512 TMEM columns
+  static constexpr int TN = T == 5 ? 128 : 96; // (T - 1) accumulators, weights 2 .. T: at most 512 TMEM columns
   static constexpr int BB = TN / 2;
   static constexpr int NACC = TN / 4;          // columns per thread (4 column groups of warps)
   static constexpr int A_SLICE = OZ_TM * OZ_KC * 2;
   static constexpr int B_SLICE = TN * OZ_KC * 2;
   static constexpr int STAGE = SA * A_SLICE + SB * B_SLICE;
-  static constexpr int SMEM = OZ_NSTAGE * STAGE + 1024 + 128;   // stages, alignment, 6 barriers + TMEM slot
+  static constexpr int SMEM = OZ_NSTAGE * STAGE + 1024 + 128;   // stages, alignment, 10 barriers + TMEM slot
   // instruction descriptor: D = F32, A = B = F16, both K-major, N = TN, M = 128
   static constexpr uint32_t IDESC = (1u << 4) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(OZ_TM >> 4) << 24);
 };
@@ -185,14 +193,18 @@ oz_outer_kernel(const float2* __restrict__ A, int nk, int nb, long long ld, long
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bar = reinterpret_cast<uint64_t*>(base + OZ_NSTAGE * O::STAGE);        // MMAs of the stage done
   uint64_t* full = bar + OZ_NSTAGE;                                                    // B slices of the stage landed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + OZ_NSTAGE * O::STAGE + 64);
-  __shared__ int s_fail;
+  uint64_t* ready = full + OZ_NSTAGE;                                                  // A slices of the stage stored
+  uint64_t* drained = ready + OZ_NSTAGE;                                               // accumulators read back
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + OZ_NSTAGE * O::STAGE + 96);
+  __shared__ volatile int s_fail;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < OZ_NSTAGE; ++i) {
       tc::mbar_init(&bar[i], 1);
       tc::mbar_init(&full[i], 1);
+      tc::mbar_init(&ready[i], OZ_WORKERS / 32);
     }
+    tc::mbar_init(drained, OZ_WORKERS / 32);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_fail = 0;
   }
@@ -206,29 +218,99 @@ oz_outer_kernel(const float2* __restrict__ A, int nk, int nb, long long ld, long
   // resident CTAs (persistent: setup, TMEM allocation and barriers once per CTA)
   const int nbt = (nb + O::BB - 1) / O::BB;
   const int ntiles = nbt * (int)((ng + OZ_TM - 1) / OZ_TM);   // < 2^31 for every supported grid
-  int bt = 0, b0 = 0, kend = 0, nchunks = 0;
-  int g0 = 0, g = 0;
-  float sa = 1.f;
+  auto kend_of = [&](int tile) {
+    const int e = (tile % nbt + 1) * O::BB;
+    return e < nk ? e : nk;
+  };
+
+  if (w >= OZ_WORKERS / 32) {            // ---------------- the issuing warp (and three idle ones)
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(OZ_REG_ISSUE));
+    if (tid == OZ_WORKERS) {
+      constexpr unsigned B_BYTES = O::SB * O::B_SLICE;
+      static_assert(B_BYTES % 16 == 0 && (O::SA * O::A_SLICE) % 16 == 0, "bulk copy alignment");
+      int ct = blockIdx.x, cc = 0, copied = 0;             // the next copy: tile, chunk of the tile, chunk of the stream
+      auto copy_b = [&]() {
+        if (ct >= ntiles) return;
+        const int s = copied % OZ_NSTAGE;
+        tc::mbar_arrive_expect_tx(&full[s], B_BYTES);
+        tc::bulk_g2s(base + s * O::STAGE + O::SA * O::A_SLICE,
+                     Bsl + (size_t)((ct % nbt) * nch + cc) * O::SB * (O::TN * OZ_KC), B_BYTES, &full[s]);
+        ++copied;
+        if (++cc == (kend_of(ct) + 15) / 16) {
+          cc = 0;
+          ct += gridDim.x;
+        }
+      };
+      auto wait = [&](uint64_t* b, int index) {            // bounded wait for completion `index` of a barrier
+        if (s_fail || !tc::mbar_wait(b, (unsigned)index & 1u, kOzWaitLimit)) {
+          s_fail = 1;
+          return false;
+        }
+        return true;
+      };
+      copy_b();
+      int n = 0, group = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        const int nchunks = (kend_of(tile) + 15) / 16;
+        for (int c = 0; c < nchunks; ++c, ++n) {
+          const int s = n % OZ_NSTAGE;
+          // the next chunk's B slices, into the stage that chunk n - 2 has left
+          if (n >= 2) ok = wait(&bar[(n + 1) % OZ_NSTAGE], (n - 2) / OZ_NSTAGE);
+          if (ok) copy_b();
+          ok = ok && wait(&ready[s], n / OZ_NSTAGE) && wait(&full[s], n / OZ_NSTAGE);
+          const bool first = c % OZ_GROUP == 0;
+          if (first) {
+            if (group > 0) ok = ok && wait(drained, group - 1);
+            ++group;
+          }
+          if (!ok) break;
+          tc::fence_after_sync();
+          // descriptors count 16-byte units; K-steps are two core matrices (256 bytes) apart
+          const uint32_t a0 = tc::smem_u32(base + s * O::STAGE);
+          const uint64_t da = tc::kmajor_desc(a0, OZ_SBO), db = tc::kmajor_desc(a0 + O::SA * O::A_SLICE, OZ_SBO);
+          uint32_t acc = tmem;
+#pragma unroll 1
+          for (int wt = 2; wt <= T; ++wt, acc += O::TN) {
+            uint64_t xa = da, xb = db + (uint64_t)((wt - 2) * (O::B_SLICE / 16));
+#pragma unroll 1
+            for (int sl = 1; sl < wt; ++sl, xa += O::A_SLICE / 16, xb -= O::B_SLICE / 16) {
+              mma_f16<T>(acc, xa, xb, first && sl == 1 ? 0u : 1u);
+              mma_f16<T>(acc, xa + 16, xb + 16, 1u);
+            }
+          }
+          tc::mma_commit(&bar[s]);
+        }
+      }
+      // bounded, also after a lost wait: the last MMAs, and copies still in flight
+      for (int i = n - OZ_NSTAGE < 0 ? 0 : n - OZ_NSTAGE; i < n; ++i)
+        if (!tc::mbar_wait(&bar[i % OZ_NSTAGE], (unsigned)(i / OZ_NSTAGE) & 1u, kOzWaitLimit)) s_fail = 1;
+      for (int i = n; i < copied; ++i)
+        if (!tc::mbar_wait(&full[i % OZ_NSTAGE], (unsigned)(i / OZ_NSTAGE) & 1u, kOzWaitLimit)) s_fail = 1;
+    }
+  } else {                               // ---------------- the working warps
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REG_WORK));
   // this thread's A elements: row r = 8 w + lane % 8, real K 4q .. 4q + 3 with q = lane / 8 and
   // q + 4, so that a warp's 8-byte slice stores cover 256 contiguous bytes (no bank conflicts)
   const int r = 8 * w + (lane & 7), q = lane >> 3;
   const uint32_t lane_col = ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(NACC * (w >> 2));
   long long acc[NACC];
 
-  auto load_a = [&](int c, float4 (&v)[2]) {
+  auto load_a = [&](int c, int kend, long long g, float4 (&v)[2]) {
+    const float2* x = A + (long long)(c * 16 + 2 * q) * ld + g;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int k = c * 16 + 2 * (q + 4 * i);
       float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
       if (g < ng) {
-        if (k < kend) { const float2 x = A[(long long)k * ld + g]; t.x = x.x; t.y = x.y; }
-        if (k + 1 < kend) { const float2 x = A[(long long)(k + 1) * ld + g]; t.z = x.x; t.w = x.y; }
+        if (k < kend) { const float2 y = x[8 * i * ld]; t.x = y.x; t.y = y.y; }
+        if (k + 1 < kend) { const float2 y = x[(8 * i + 1) * ld]; t.z = y.x; t.w = y.y; }
       }
       v[i] = t;
     }
   };
   // the SA slices of this thread's 8 values into stage `st`
-  auto store_a = [&](unsigned char* st, const float4 (&v)[2]) {
+  auto store_a = [&](unsigned char* st, const float4 (&v)[2], float sa) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       float x[4] = {v[i].x * sa, v[i].y * sa, v[i].z * sa, v[i].w * sa};
@@ -249,154 +331,96 @@ oz_outer_kernel(const float2* __restrict__ A, int nk, int nb, long long ld, long
       }
     }
   };
-  constexpr unsigned B_BYTES = O::SB * O::B_SLICE;
-  static_assert(B_BYTES % 16 == 0 && (O::SA * O::A_SLICE) % 16 == 0, "bulk copy alignment");
-  auto copy_b = [&](unsigned char* st, int c, int s) {   // thread 0
-    tc::mbar_arrive_expect_tx(&full[s], B_BYTES);
-    tc::bulk_g2s(st + O::SA * O::A_SLICE, Bsl + (size_t)(bt * nch + c) * O::SB * (O::TN * OZ_KC), B_BYTES, &full[s]);
-  };
-  auto issue = [&](const unsigned char* st, bool group_first) {
-    const uint32_t a0 = tc::smem_u32(st), bb0 = a0 + O::SA * O::A_SLICE;
-    bool first[O::NW];
-#pragma unroll
-    for (int i = 0; i < O::NW; ++i) first[i] = group_first;
-#pragma unroll
-    for (int wt = 2; wt <= T; ++wt) {
-#pragma unroll
-      for (int s = 1; s <= O::SA; ++s) {
-        const int t = wt - s;
-        if (t < 1 || t > O::SB) continue;
-#pragma unroll
-        for (int ks = 0; ks < OZ_KC / 16; ++ks) {
-          const uint32_t o = ks * 256;    // two core matrices of 16 B along K per K-step of 16
-          mma_f16<T>(tmem + (uint32_t)((wt - 2) * O::TN), tc::kmajor_desc(a0 + (s - 1) * O::A_SLICE + o, OZ_SBO),
-                     tc::kmajor_desc(bb0 + (t - 1) * O::B_SLICE + o, OZ_SBO), first[wt - 2] ? 0u : 1u);
-          first[wt - 2] = false;
-        }
-      }
-    }
-  };
   auto drain = [&]() {
     tc::fence_after_sync();
 #pragma unroll
     for (int wt = 2; wt <= T; ++wt) {
       const uint32_t ta = tmem + lane_col + (uint32_t)((wt - 2) * O::TN);
       const int sh = OZ_BETA * (T - wt);
-      uint32_t v[32];
-      if constexpr (NACC == 32) {
-        tc::tmem_ld32(ta, v);
-      } else {
-        tc::tmem_ld16(ta, v);
-        tc::tmem_ld8(ta + 16, v + 16);
-      }
-      tc::tmem_wait_ld();
 #pragma unroll
-      for (int j = 0; j < NACC; ++j) acc[j] += (long long)__float2int_rn(__uint_as_float(v[j])) << sh;
+      for (int o = 0; o < NACC; o += 8) {                  // eight at a time: the sums hold half of the registers
+        uint32_t v[8];
+        tc::tmem_ld8(ta + (uint32_t)o, v);
+        tc::tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[o + j] += (long long)__float2int_rn(__uint_as_float(v[j])) << sh;
+      }
     }
     tc::fence_before_sync();
   };
 
-  // Thread 0 alone waits on the barriers: the MMA commits (bit s of `issued`:
-  // a commit on stage s not yet seen) and the bulk copies (`inflight`).
-  unsigned phase = 0, issued = 0;
-  unsigned fphase = 0, inflight = 0;
-  bool ok = true;
-  auto landed = [&](int s) -> bool {   // bounded wait for the bulk copy into stage s
-    if (!tc::mbar_wait(&full[s], (fphase >> s) & 1u, kOzWaitLimit)) return false;
-    fphase ^= 1u << s;
-    inflight &= ~(1u << s);
-    return true;
+  auto wait = [&](int n) {               // bounded wait for the MMAs of chunk n of the stream
+    if (!tc::mbar_wait(&bar[n % OZ_NSTAGE], (unsigned)(n / OZ_NSTAGE) & 1u, kOzWaitLimit)) s_fail = 1;
+    return !s_fail;
   };
-  auto settle = [&](int s) -> bool {   // bounded wait for the MMAs last committed on stage s
-    if (!tc::mbar_wait(&bar[s], (phase >> s) & 1u, kOzWaitLimit)) return false;
-    phase ^= 1u << s;
-    issued &= ~(1u << s);
-    return true;
+  auto arrive = [&](uint64_t* b) {       // one arrival per warp, after all its lanes
+    __syncwarp();
+    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(b)) : "memory");
   };
-  float4 cur[2], nxt[2];
-  int cc = 0;                          // chunks issued by this CTA (stage rotation)
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    bt = tile % nbt;
-    b0 = bt * O::BB;
-    g0 = (tile / nbt) * OZ_TM;
-    kend = b0 + O::BB < nk ? b0 + O::BB : nk;
-    nchunks = (kend + 15) / 16;
-    g = g0 + r;
-    sa = ldexpf(1.0f, OZ_BETA - (g < ng ? erow[g] : 0));   // exact power of two
+  auto output = [&](int tile) {          // a finished tile, then zero sums
+    const int row = 32 * (w & 3) + lane, b0 = (tile % nbt) * O::BB;
+    const long long gg = (long long)(tile / nbt) * OZ_TM + row;
+    const int ri = (w >> 2) >= 2 ? 1 : 0;                 // column groups 0-1 real, 2-3 imaginary
+    const int jq = ((w >> 2) & 1) * NACC;
+    if (gg < ng) {
+      const int ergg = erow[gg];
+#pragma unroll
+      for (int j = 0; j < NACC; ++j) {
+        const int b = b0 + jq + j;
+        if (b < nb) {
+          const int e = ergg + fcol[b] - OZ_BETA * T;
+          if constexpr (sizeof(OUT) == 8)   // one rounding of the exact integer, then an exact power of two
+            reinterpret_cast<float*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexpf(__ll2float_rn(acc[j]), e);
+          else
+            reinterpret_cast<double*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexp(__ll2double_rn(acc[j]), e);
+        }
+        if (j % 4 == 3) asm volatile("" ::: "memory");     // a few loads at a time: registers are short
+      }
+    }
 #pragma unroll
     for (int j = 0; j < NACC; ++j) acc[j] = 0;
-    if (nchunks > 0) load_a(0, cur);
-    for (int c = 0; c < nchunks; ++c, ++cc) {
-      // stage s is free: thread 0 saw its previous MMAs (chunk cc - 3) complete
-      // before the barrier of chunk cc - 1, or at the last drain
-      const int s = cc % OZ_NSTAGE;
-      unsigned char* st = base + s * O::STAGE;
-      if (c + 1 < nchunks) load_a(c + 1, nxt);
-      if (tid == 0) {
-        copy_b(st, c, s);
-        inflight |= 1u << s;
-      }
-      store_a(st, cur);
-      tc::fence_async_smem();
-      if (tid == 0) {                  // the stage the next chunk writes: its MMAs (chunk cc - 2)
-        const int sn = (s + 1) % OZ_NSTAGE;
-        if (((issued >> sn) & 1u) && !settle(sn)) s_fail = 1;
-      }
-      __syncthreads();
-      if (s_fail) { ok = false; break; }
-      if (tid == 0) {
-        if (landed(s)) {
-          tc::fence_after_sync();
-          issue(st, (c % OZ_GROUP) == 0);
-          tc::mma_commit(&bar[s]);
-          issued |= 1u << s;
-        } else {
-          s_fail = 1;                  // seen by every thread after the next barrier
-        }
-      }
-      if ((c % OZ_GROUP) == OZ_GROUP - 1 || c == nchunks - 1) {
-        // thread 0 sees every MMA so far complete, then all threads drain
-        if (tid == 0 && !s_fail)
-          for (int i = 0; i < OZ_NSTAGE; ++i)
-            if (((issued >> i) & 1u) && !settle(i)) s_fail = 1;
-        __syncthreads();
-        if (s_fail) { ok = false; break; }
-        drain();
-      }
-      cur[0] = nxt[0];
-      cur[1] = nxt[1];
-    }
-    if (!ok) break;
-    {   // the tile's outputs
-      const int row = 32 * (w & 3) + lane;
-      const long long gg = g0 + row;
-      const int ergg = gg < ng ? erow[gg] : 0;
-      const int ri = (w >> 2) >= 2 ? 1 : 0;                 // column groups 0-1 real, 2-3 imaginary
-      const int jq = ((w >> 2) & 1) * NACC;
-      if (gg < ng) {
+  };
+  float4 cur[2];
+  int n = 0, due = -1;                   // chunk of the stream; tile that ends with the pending group
+  bool pending = false, ok = true;       // a group ended with chunk n - 1
 #pragma unroll
-        for (int j = 0; j < NACC; ++j) {
-          const int b = b0 + jq + j;
-          if (b < nb) {
-            const int e = ergg + fcol[b] - OZ_BETA * T;
-            if constexpr (sizeof(OUT) == 8)   // one rounding of the exact integer, then an exact power of two
-              reinterpret_cast<float*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexpf(__ll2float_rn(acc[j]), e);
-            else
-              reinterpret_cast<double*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexp(__ll2double_rn(acc[j]), e);
-          }
-        }
-      }
-    }
-  }   // tiles
-  // commits and bulk copies still outstanding (bounded; also after a lost wait)
-  if (tid == 0) {
-    for (int i = 0; i < OZ_NSTAGE; ++i)
-      if (((issued >> i) & 1u) && !settle(i)) s_fail = 1;
-    for (int i = 0; i < OZ_NSTAGE; ++i)
-      if (((inflight >> i) & 1u) && !landed(i)) s_fail = 1;
+  for (int j = 0; j < NACC; ++j) acc[j] = 0;
+  int next_e = 0;                        // exponent of this thread's row in the next tile
+  if ((int)blockIdx.x < ntiles) {
+    const long long g = (long long)(blockIdx.x / nbt) * OZ_TM + r;
+    load_a(0, kend_of(blockIdx.x), g, cur);
+    next_e = g < ng ? erow[g] : 0;
   }
+  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    const int kend = kend_of(tile), nchunks = (kend + 15) / 16, next = tile + gridDim.x;
+    const long long g = (long long)(tile / nbt) * OZ_TM + r, gn = (long long)(next / nbt) * OZ_TM + r;
+    const float sa = ldexpf(1.0f, OZ_BETA - next_e);       // exact power of two
+    if (next < ntiles) next_e = gn < ng ? erow[gn] : 0;
+    for (int c = 0; c < nchunks; ++c, ++n) {
+      const bool last = c == nchunks - 1;
+      if (n >= OZ_NSTAGE && !wait(n - OZ_NSTAGE)) { ok = false; break; }
+      store_a(base + (n % OZ_NSTAGE) * O::STAGE, cur, sa);
+      tc::fence_async_smem();
+      arrive(&ready[n % OZ_NSTAGE]);
+      if (!last) load_a(c + 1, kend, g, cur);
+      else if (next < ntiles) load_a(0, kend_of(next), gn, cur);
+      if (pending) {
+        if (!wait(n - 1)) { ok = false; break; }
+        drain();
+        arrive(drained);
+        if (due >= 0) output(due);
+      }
+      pending = last || c % OZ_GROUP == OZ_GROUP - 1;
+      due = last ? tile : -1;
+    }
+  }
+  if (ok && pending && wait(n - 1)) {
+    drain();
+    output(due);
+  }
+  }   // working warps
   __syncthreads();
-  if ((!ok || s_fail) && tid == 0) {
+  if (s_fail && tid == 0) {
     status[0] = -6;   // ACE_ERR_TIMEOUT
     status[1] = -3;
   }
