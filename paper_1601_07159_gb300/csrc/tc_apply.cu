@@ -17,7 +17,7 @@
 //          BB + j take (im, -re).
 //   outer: rows g, K' = 2 N; columns j < BB take (Re C, -Im C), BB + j (Im C, Re C).
 //
-// Pipeline (512 threads, one CTA per SM, M = 128): K runs in chunks of 32 real terms.
+// Pipeline (512 working threads, one CTA per SM, M = 128): K runs in chunks of 32 real terms.
 // One thread keeps a ring of raw FP32 chunks filled by TMA, as deep as shared
 // memory allows; every thread converts eight values of one row (A), or of one row of A and
 // one of B, from the ring into an operand stage (K-major core matrices,
@@ -33,7 +33,7 @@
 //
 // Measured, TF32 split -> this: 48^3, 128 orbitals, 192 bands: gram 169 -> 94 us, outer
 // 188 -> 122 us, the new pass over the vectors for their largest values 48 us (5.9
-// TB/s), whole call 378 -> 299 us; 96^3, 1024 x 1536: 116 -> 79 ms (gram 38,
+// TB/s), whole call 378 -> 294 us; 96^3, 1024 x 1536: 116 -> 79 ms (gram 38,
 // outer 39). With the MMAs and the conversion switched off the 48^3 loops still take 67
 // and 95 us (387 and 553 MB through L2, 5.8 TB/s): tile traffic bounds them, then the
 // chain convert - fence - barrier - issue of a chunk. Relative error against FP64 at
@@ -71,6 +71,12 @@ template <int TN> struct Tile {
   // gram: stages of A_hi, A_lo, B_hi, B_lo and a raw ring of A and B rows
   static constexpr int G_STAGE = 2 * A_TILE + 2 * B_TILE;
   static constexpr int G_RAW = (TM + BB) * KC * 4;
+  // The narrow tiles' chunks are short beside a block-wide barrier and the issue of their
+  // MMAs: a warp of its own fetches and issues, and the working warps meet it on
+  // mbarriers (16 x 24 vectors of 48^3: 38.0 us without, 35.6 us with). The wide ones need
+  // the registers that a fifth warp per SM quadrant takes.
+  static constexpr bool G_ISSUER = TN <= 128;
+  static constexpr int G_THREADS = THREADS + (G_ISSUER ? 128 : 0);
   static constexpr int G_STAGES = TN == 64 ? 4 : TN == 256 ? 2 : 3;
   static constexpr int G_RING = TN == 64 ? 6 : TN == 128 ? 5 : TN == 192 ? 3 : 4;   // what 227 KB hold
   static constexpr int G_SMEM = G_STAGES * G_STAGE + G_RING * G_RAW + 1024 + 128;
@@ -133,16 +139,19 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b,
       : "memory");
 }
 
-// the MMAs of one chunk: 2 K-steps x 3 products
+// the MMAs of one chunk: 2 K-steps x 3 products. Descriptors count 16-byte units, so
+// the operands' are sums with constants: one thread issues, and the block's
+// other warps wait for its warp.
 template <int TN>
 __device__ __forceinline__ void issue_chunk(uint32_t dtmem, uint32_t a, uint32_t b, bool first) {
-  const uint32_t al = a + A_TILE, bl = b + Tile<TN>::B_TILE;
+  const uint64_t ah = tc::kmajor_desc(a, SBO), bh = tc::kmajor_desc(b, SBO);
+  constexpr uint64_t LA = A_TILE / 16, LB = Tile<TN>::B_TILE / 16;
 #pragma unroll
-  for (int ks = 0; ks < KC / 16; ++ks) {
-    const uint32_t o = ks * 256;   // two core matrices of 16 bytes along K
-    mma_f16<TN>(dtmem, tc::kmajor_desc(a + o, SBO), tc::kmajor_desc(b + o, SBO), (first && ks == 0) ? 0u : 1u);
-    mma_f16<TN>(dtmem, tc::kmajor_desc(a + o, SBO), tc::kmajor_desc(bl + o, SBO), 1u);
-    mma_f16<TN>(dtmem, tc::kmajor_desc(al + o, SBO), tc::kmajor_desc(b + o, SBO), 1u);
+  for (uint64_t ks = 0; ks < KC / 16; ++ks) {
+    const uint64_t o = ks * 16;   // two core matrices of 16 bytes along K
+    mma_f16<TN>(dtmem, ah + o, bh + o, (first && ks == 0) ? 0u : 1u);
+    mma_f16<TN>(dtmem, ah + o, bh + LB + o, 1u);
+    mma_f16<TN>(dtmem, ah + LA + o, bh + o, 1u);
   }
 }
 
@@ -199,16 +208,17 @@ template <int TN> struct Stream {
 };
 
 template <int TN>
-__device__ __forceinline__ uint32_t setup(uint64_t* bar, int nbar, uint32_t* slot) {
+__device__ __forceinline__ uint32_t setup(uint64_t* bar, int nbar, uint32_t* slot, int nwarps = 0) {
   if (threadIdx.x == 0) {
     for (int i = 0; i < nbar; ++i) tc::mbar_init(&bar[i], 1);
+    for (int i = 0; i < nwarps; ++i) tc::mbar_init(&bar[nbar + i], THREADS / 32);   // one arrival per working warp
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x < 32) tc::tmem_alloc_warp(slot, Tile<TN>::TMEM_COLS);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  return *slot;
+  return __shfl_sync(0xffffffffu, *slot, 0);   // the same register for the whole warp
 }
 template <int TN> __device__ __forceinline__ void teardown(uint32_t tmem) {
   tc::fence_before_sync();
@@ -257,7 +267,7 @@ vec_max_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ 
 // loads. Thread t owns row 8 (t / 32) + t % 8 and granules q and q + 4, q = (t / 8) % 4:
 // its loads are conflict-free and its stores fill 128 contiguous bytes per 16 lanes.
 template <int TN>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(Tile<TN>::G_THREADS, 1)
 gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_constant__ CUtensorMap B, int nb, long long ng,
               const unsigned* __restrict__ mx, float2* __restrict__ part, long long chunk, int* status) {
   using T = Tile<TN>;
@@ -265,15 +275,15 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* ring = base + ST * T::G_STAGE;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ring + R * T::G_RAW);   // [0, ST): MMAs of a stage; then R: a chunk landed
-  __shared__ int s_fail;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(ring + R * T::G_RAW);   // [0, ST): MMAs of a stage; then R: a chunk landed; then ST: a stage stored
+  __shared__ volatile int s_fail;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   if (tid == 0) s_fail = 0;
   Stream<TN> S;
   S.bar = bar;
-  S.tmem = setup<TN>(bar, ST + R, reinterpret_cast<uint32_t*>(bar + ST + R));
+  constexpr bool IW = T::G_ISSUER;
+  S.tmem = setup<TN>(bar, ST + R, reinterpret_cast<uint32_t*>(bar + 2 * ST + R), IW ? ST : 0);
   S.lane_col = ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(NH * (w >> 2));
-  S.zero();
 
   const int a0 = blockIdx.x * TM, b0 = blockIdx.y * BB;
   const long long g_begin = (long long)blockIdx.z * chunk;
@@ -293,8 +303,33 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
       load_box(d + TM * KC * 4, B, x, b0, fb);
     }
   };
-  if (tid == 32)
+  if (IW && w >= THREADS / 32) {                         // ---- the issuing warp (and three idle ones)
+    if (TN == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
+    if (tid == THREADS) {
+      int c = 0;
+      for (int i = 0; i < R; ++i) fetch(i);
+      for (; c < nchunks; ++c) {
+        const int s = c % ST;
+        // stored by all warps: also read from the ring, and the sums of the group that
+        // last used this chunk's accumulator are drained (their stage came before)
+        if (!tc::mbar_wait(bar + ST + R + s, (unsigned)(c / ST) & 1u, kWaitLimit)) break;
+        tc::fence_after_sync();
+        const uint32_t sa0 = smem_u32(base + s * T::G_STAGE);
+        issue_chunk<TN>(S.tmem + (uint32_t)(TN * ((c / kGroup) & 1)), sa0, sa0 + 2 * A_TILE, c % kGroup == 0);
+        tc::mma_commit(&bar[s]);
+        fetch(c + R);
+      }
+      if (c < nchunks) {                                 // a lost wait: the copies and MMAs in flight (bounded)
+        s_fail = 1;
+        for (int i = c; i < c + R && i < nchunks; ++i) tc::mbar_wait(bar + ST + i % R, (unsigned)(i / R) & 1u, 1u << 16);
+        for (int i = c < ST ? 0 : c - ST; i < c; ++i) tc::mbar_wait(&bar[i % ST], (unsigned)(i / ST) & 1u, 1u << 16);
+      }
+    }
+  } else {                                               // ---- the working warps
+  if (TN == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");   // 512 x 112 + 128 x 24 of 640 x 96 registers
+  if (!IW && tid == 32)
     for (int c = 0; c < R - 1; ++c) fetch(c);
+  S.zero();
   const int o = tile_off(r, 4 * q);
   constexpr int IM = (BB >> 3) * SBO;                    // rows BB ..: (im, -re)
   const int g0 = r * 128 + ((q ^ (r & 7)) << 4), g1 = g0 ^ 64;   // the granules in a raw tile
@@ -302,7 +337,7 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
   unsigned lphase = 0;                                   // parities of the landing barriers
   for (int c = 0; c < nchunks; ++c) {
     const int s = c % ST, slot = c % R;
-    if (tid == 32) fetch(c + R - 1);                     // into the slot that chunk c - 1 left
+    if (!IW && tid == 32) fetch(c + R - 1);               // into the slot that chunk c - 1 left
     if (!tc::mbar_wait(bar + ST + slot, (lphase >> slot) & 1u, kWaitLimit)) s_fail = 1;
     else lphase ^= 1u << slot;
     const unsigned char* raw = ring + slot * T::G_RAW;
@@ -331,17 +366,27 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
       }
     }
     tc::fence_async_smem();
-    __syncthreads();
-    if (s_fail) {
-      ok = false;
-      break;
-    }
     const int buf = (c / kGroup) & 1;
-    if (tid == 0) {
-      const uint32_t sa0 = smem_u32(base + s * T::G_STAGE);
-      tc::fence_after_sync();
-      issue_chunk<TN>(S.tmem + (uint32_t)(TN * buf), sa0, sa0 + 2 * A_TILE, c % kGroup == 0);
-      tc::mma_commit(&bar[s]);
+    if constexpr (IW) {
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar + ST + R + s)) : "memory");
+      if (s_fail) {
+        ok = false;
+        break;
+      }
+    } else {
+      __syncthreads();
+      if (s_fail) {
+        ok = false;
+        break;
+      }
+      if (tid == 0) {
+        const uint32_t sa0 = smem_u32(base + s * T::G_STAGE);
+        tc::fence_after_sync();
+        issue_chunk<TN>(S.tmem + (uint32_t)(TN * buf), sa0, sa0 + 2 * A_TILE, c % kGroup == 0);
+        tc::mma_commit(&bar[s]);
+      }
     }
     S.issued |= 1u << s;
     if (c % kGroup == kGroup - 1 || c == nchunks - 1) S.drain |= (1u + (unsigned)buf) << (2 * s);
@@ -350,20 +395,21 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
     const int s = (nchunks + i) % ST;
     if (((S.issued >> s) & 1u) && !S.settle(s)) s_fail = 1;
   }
-  if (!ok)                                               // copies in flight (bounded)
+  if (!IW && !ok)                                        // copies in flight (bounded)
     for (int i = 0; i < R; ++i) tc::mbar_wait(bar + ST + i, (lphase >> i) & 1u, 1u << 16);
-  __syncthreads();
-  ok = ok && !s_fail;
-  if (!ok && tid == 0) {
-    status[0] = -6;   // ACE_ERR_TIMEOUT
-    status[1] = -4;
-  }
   const int a = a0 + 32 * (w & 3) + lane, bq = b0 + NH * (w >> 2);
   if (ok && a < na) {
     float2* out = part + ((long long)blockIdx.z * na + a) * nb + bq;
 #pragma unroll
     for (int j = 0; j < NH; ++j)
       if (bq + j < nb) out[j] = make_float2(S.re[j], S.im[j]);
+  }
+  if (!ok) s_fail = 1;
+  }   // working warps
+  __syncthreads();
+  if (s_fail && tid == 0) {
+    status[0] = -6;   // ACE_ERR_TIMEOUT
+    status[1] = -4;
   }
   teardown<TN>(S.tmem);
 }
@@ -772,7 +818,7 @@ int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld
     constexpr int TN = decltype(t)::value;
     using T = Tile<TN>;
     const int nbt = (nb + T::BB - 1) / T::BB;
-    gram16_kernel<TN><<<dim3((n + TM - 1) / TM, nbt, splits), THREADS, T::G_SMEM, st>>>(xg, n, qg, nb, ng, s.mx, s.part,
+    gram16_kernel<TN><<<dim3((n + TM - 1) / TM, nbt, splits), T::G_THREADS, T::G_SMEM, st>>>(xg, n, qg, nb, ng, s.mx, s.part,
                                                                                      chunk, status);
     const long long total = (long long)n * nb;
     int ways = 8;
