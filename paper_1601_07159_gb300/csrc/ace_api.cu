@@ -351,7 +351,8 @@ WsLayout layout(const ace_plan* p, int op, int nb, char* base) {
   if (op == ACE_OP_APPLY) {
     L.part = (double*)take((size_t)splits * N * nb * 2 * sizeof(double));
     L.Cm = (double*)take((size_t)N * nb * 2 * sizeof(double));
-    if (p->apply16 && nb > 0 && off < apply_tc_scratch_bytes(p->ng, N, nb)) off = apply_tc_scratch_bytes(p->ng, N, nb);
+    // a few bands or orbitals: the FP16 products' padded right operand is the larger
+    if (p->apply16 && nb > 0 && off < apply_tc_least_bytes(p->ng, N, nb)) off = apply_tc_least_bytes(p->ng, N, nb);
   }
   L.total = off;
   return L;
@@ -1422,7 +1423,7 @@ ace_status ace_apply(ace_plan* p, const void* Xi, const void* Psi, int nb, void*
   const WsLayout Wl = layout(p, ACE_OP_APPLY, nb, (char*)ws);
   // C = dV Xi^* Psi, Y = -Xi C (Eq. ACE)
   if (p->apply16 && apply_tc_faster(p->ng, N, nb)) {
-    const int k = launch_apply_tc(Xi, N, Psi, nb, p->ld, p->ng, p->dv, Y, ws, p->status, st);
+    const int k = launch_apply_tc(Xi, N, Psi, nb, p->ld, p->ng, p->dv, Y, ws, Wl.total, p->status, st);
     if (k == 0) return fail(ACE_ERR_CUDA, "tensor map encoding failed");
     p->launches += k;
     return cuda_check("ace_apply");

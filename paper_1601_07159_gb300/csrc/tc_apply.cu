@@ -703,13 +703,14 @@ template <typename F> void by_width(int tn, F&& f) {
 }
 
 // Split-K count of the gram product: fewest waves per split, within 2 % of full waves
-// if that can be had (the fewest such splits: each adds partial sums).
-int splits_for(long long ng, int na, int nb) {
+// if that can be had (the fewest such splits: each adds partial sums), at most `cap`.
+int splits_for(long long ng, int na, int nb, long long cap) {
   constexpr long long kSMs = 152, kMaxSplits = 1024;
   const int bb = width(nb) / 2;
   const long long tiles = (long long)((na + TM - 1) / TM) * ((nb + bb - 1) / bb);
   long long max_s = (ng + KC / 2 - 1) / (KC / 2);
   if (max_s > kMaxSplits) max_s = kMaxSplits;
+  if (max_s > cap) max_s = cap;
   long long best = 1;
   double best_cost = (double)((tiles + kSMs - 1) / kSMs);
   for (long long waves = 1; best_cost > 1.02 * tiles / kSMs; ++waves) {   // the most splits of each wave count
@@ -727,16 +728,19 @@ int splits_for(long long ng, int na, int nb) {
 }
 
 // Scratch layout: vector maxima, column scales, C, and the split sums, which the right
-// operand overwrites once they are reduced.
+// operand overwrites once they are reduced. The splits are those that fit `budget`
+// bytes (the plan's workspace is sized by the TF32 products, so that it does not depend on
+// a call's path); least = bytes for one.
 struct Scratch {
   unsigned* mx;
   float2* colscale;
   unsigned char* Bs;
   float2* C;
   float2* part;
-  size_t total;
+  int splits;
+  size_t least;
 };
-Scratch scratch(char* base, long long ng, int n, int nb) {
+Scratch scratch(char* base, long long ng, int n, int nb, size_t budget) {
   Scratch s{};
   size_t off = 0;
   auto take = [&](size_t bytes) { char* r = base ? base + off : nullptr; off += align256(bytes); return r; };
@@ -745,10 +749,11 @@ Scratch scratch(char* base, long long ng, int n, int nb) {
   s.mx = (unsigned*)take((size_t)(n + nb) * sizeof(unsigned));
   s.colscale = (float2*)take((size_t)nb * sizeof(float2));
   s.C = (float2*)take((size_t)n * nb * sizeof(float2));
-  const size_t pb = (size_t)splits_for(ng, n, nb) * n * nb * sizeof(float2), bs = nbt * nch * (size_t)(2 * bb) * KC * 2 * 2;
-  s.part = (float2*)take(pb > bs ? pb : bs);
+  s.part = (float2*)take(0);
   s.Bs = (unsigned char*)s.part;
-  s.total = off;
+  const size_t one = (size_t)n * nb * sizeof(float2), bs = nbt * nch * (size_t)(2 * bb) * KC * 2 * 2;
+  s.least = off + align256(one > bs ? one : bs);
+  if (s.least <= budget) s.splits = splits_for(ng, n, nb, (long long)((budget - off) / one));
   return s;
 }
 
@@ -796,12 +801,13 @@ bool apply_tc_faster(long long ng, int n, int nb) {
   return ng >= (1LL << 16) || ng * ((long long)n + nb) >= (7LL << 18);
 }
 
-size_t apply_tc_scratch_bytes(long long ng, int n, int nb) { return scratch(nullptr, ng, n, nb).total; }
+size_t apply_tc_least_bytes(long long ng, int n, int nb) { return scratch(nullptr, ng, n, nb, 0).least; }
 
 int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld, long long ng, double dv, void* Y,
-                    void* ws, int* status, cudaStream_t st) {
-  const Scratch s = scratch(static_cast<char*>(ws), ng, n, nb);
+                    void* ws, size_t budget, int* status, cudaStream_t st) {
+  const Scratch s = scratch(static_cast<char*>(ws), ng, n, nb, budget);
   const float2 *x = static_cast<const float2*>(Xi), *psi = static_cast<const float2*>(Psi);
+  if (s.splits < 1) return 0;
   CUtensorMap xg, qg, xo;                 // Xi and Psi of the gram product, Xi of the outer one
   if (!encoder() || !vector_map(&xg, x, n, ld, ng, KC / 2, TM, true) ||
       !vector_map(&qg, psi, nb, ld, ng, KC / 2, width(nb) / 2, true) || !vector_map(&xo, x, n, ld, ng, TM, KC / 2, false))
@@ -811,7 +817,7 @@ int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld
   long long per = (16 * 152 + n + nb - 1) / (n + nb), most = (ng / 2 + 1023) / 1024;
   per = per < 1 ? 1 : per > most ? most : per;
   vec_max_kernel<<<dim3(n + nb, (unsigned)per), 256, 0, st>>>(x, n, psi, ld, ng, s.mx);
-  const int splits = splits_for(ng, n, nb), nch = (n + 15) / 16;
+  const int splits = s.splits, nch = (n + 15) / 16;
   long long chunk = (ng + splits - 1) / splits;
   chunk = (chunk + KC / 2 - 1) / (KC / 2) * (KC / 2);
   by_width(width(nb), [&](auto t) {

@@ -2,7 +2,8 @@
 edges of its tiles: orbital counts around the 16 of a K chunk and the 128 of a
 row tile, band counts that take each MMA width (64, 128, 192 and 256 columns) and
 leave a partial last tile, a point count that is not a multiple of 128,
-padded vectors, vectors of very different scales, one call below the line; against
+padded vectors, vectors of very different scales, one call below the line, one whose
+splits the workspace bounds; against
 the oracle and the TF32-split apply.
 
 Tolerance: operands keep 22 bits (2^-23 rounding) of every value down to 2^-18 of
@@ -22,7 +23,8 @@ TOL = 1e-5
 
 CASES = [((48, 48, 48), 16, 24, 0), ((48, 48, 48), 1, 1, 0), ((48, 48, 48), 17, 33, 0), ((48, 48, 48), 130, 3, 2), ((36, 36, 36), 1, 97, 0),
          ((36, 36, 36), 33, 96, 6), ((20, 20, 36), 100, 200, 0), ((48, 40, 36), 128, 129, 0), ((32, 32, 32), 15, 200, 0),
-         ((24, 24, 24), 20, 30, 0)]
+         ((24, 24, 24), 20, 30, 0),
+         ((36, 36, 36), 300, 300, 0)]
 
 
 @pytest.fixture(scope="module")
