@@ -520,8 +520,10 @@ outer_tc_kernel(const float2* __restrict__ A, int nk, const float2* __restrict__
 }
 
 // Exact diagonal of the gram product: Mc[a][a] = (scale Re sum_g conj(A_a) B_a, 0),
-// FP32 products summed in FP32 over short runs and in FP64 across them.
-// Grid: (na, splits), splits <= kDiagSplits; part: FP64 [na][kDiagSplits].
+// FP32 products summed in FP32 over runs of 16 points a thread and in FP64 across them.
+// Memory-bound once eight points of both vectors are in flight per thread (one at a
+// time: 68 us for 128 orbitals of 48^3, 226 MB; 40 us so); points past the split's
+// end add zeros. Grid: (na, splits), splits <= kDiagSplits; part: FP64 [na][kDiagSplits].
 constexpr int kDiagSplits = 32;
 __global__ void __launch_bounds__(256)
 diag_dot_kernel(const float2* __restrict__ A, const float2* __restrict__ B, long long ld, long long ng,
@@ -530,15 +532,24 @@ diag_dot_kernel(const float2* __restrict__ A, const float2* __restrict__ B, long
   const int a = blockIdx.x;
   const long long per = (ng + gridDim.y - 1) / gridDim.y;
   const long long g0 = blockIdx.y * per, g1 = g0 + per < ng ? g0 + per : ng;
+  const float2 *pa = A + (long long)a * ld, *pb = B + (long long)a * ld;
   double s = 0.0;
-  float run = 0.f;
-  int cnt = 0;
-  for (long long g = g0 + threadIdx.x; g < g1; g += blockDim.x) {
-    const float2 x = A[(long long)a * ld + g], y = B[(long long)a * ld + g];
-    run = fmaf(x.x, y.x, fmaf(x.y, y.y, run));
-    if (++cnt == 16) { s += (double)run; run = 0.f; cnt = 0; }
+  for (long long g = g0 + threadIdx.x; g < g1; g += 16 * 256) {
+    float run = 0.f;
+#pragma unroll
+    for (int h = 0; h < 16; h += 8) {
+      float2 x[8], y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const long long q = g + (h + i) * 256;
+        x[i] = q < g1 ? pa[q] : make_float2(0.f, 0.f);
+        y[i] = q < g1 ? pb[q] : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) run = fmaf(x[i].x, y[i].x, fmaf(x[i].y, y[i].y, run));
+    }
+    s += (double)run;
   }
-  s += (double)run;
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();

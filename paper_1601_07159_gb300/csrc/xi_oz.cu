@@ -124,6 +124,7 @@ __global__ void oz_row_exp_kernel(const float2* __restrict__ A, int nk, long lon
                                   int* __restrict__ erow) {
   for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += (long long)gridDim.x * blockDim.x) {
     float m = 0.f;
+#pragma unroll 8
     for (int k = 0; k < nk; ++k) {
       const float2 v = A[(long long)k * ld + g];
       m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
