@@ -448,6 +448,7 @@ long long issue_pairs(ace_plan* p, const PairLaunch& base, const Schedule& sc, c
       L.Epart = E0;
       L.ev = take_events(p, 5, 0);
       L.dtiles = sc.dtiles + sc.toff[k];
+      L.lead = k == 0;
       L.clear = clear_in_a && k == 0 ? p->status : nullptr;
       kernels += launches(gmask, L.mode);
       if (!launch_one(p, L, b, cs)) return -1;
@@ -469,6 +470,7 @@ long long issue_pairs(ace_plan* p, const PairLaunch& base, const Schedule& sc, c
       L.Epart = E0;
       L.ev = nullptr;
       L.dtiles = sc.dtiles + sc.toff[k];
+      L.lead = k == 0;
       L.clear = clear_in_a && k == 0 ? p->status : nullptr;
       ok = ok && launch_one(p, L, sc.batches[k], cs);
       kernels += launches(gmask, L.mode);
@@ -494,6 +496,7 @@ long long issue_pairs(ace_plan* p, const PairLaunch& base, const Schedule& sc, c
       L.Epart = E0;
       L.ev = nullptr;
       L.dtiles = sc.dtiles + sc.toff[k];
+      L.lead = k == 0;
       L.pass_mask = 1 & gmask;
       if (L.pass_mask) ok = ok && launch_one(p, L, sc.batches[k], la);
       cudaEventRecord(p->ov_ev[0], la);
@@ -539,6 +542,7 @@ long long issue_pairs(ace_plan* p, const PairLaunch& base, const Schedule& sc, c
     L.Epart = E0 ? E0 + (size_t)ln * epart_per_lane(p) : nullptr;
     L.ev = nullptr;
     L.dtiles = sc.dtiles + sc.toff[k];
+    L.lead = k == 0;
     kernels += launches(gmask, L.mode);
     ok = ok && launch_one(p, L, sc.batches[k], p->lane[ln]);
   }

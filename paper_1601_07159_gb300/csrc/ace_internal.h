@@ -62,6 +62,7 @@ struct PairLaunch {
   bool prepare_only;     // set kernel attributes for edge n, launch nothing
   const TileDesc* dtiles;  // device copy of the batch's tile descriptors
   bool no_pdl;           // launch the passes without programmatic dependent launch
+  bool lead;             // the call's first batch: its pass A is launched without it (X, Y are the caller's work)
   int pass_mask;         // passes to launch: bit 0 A, 1 B, 2 C, 3 D (0 = all)
   int radix;             // line-transform radix order: 0 radix 4 first, 1 odd radix first (FP32)
 };

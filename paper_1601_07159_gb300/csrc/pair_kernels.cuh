@@ -131,6 +131,10 @@ template <typename R> struct PointParams {
 // programmatic stream serialisation, so its blocks take the slots that the
 // previous pass's last blocks leave; griddep_wait() blocks until the previous
 // grid has completed and its writes are visible (a no-op without the attribute).
+// Pass A reads X and Y before it waits: none of the passes writes them. The kernel in
+// front of a call's first pass A may have (an eager call on vectors that the
+// caller's last kernel wrote), so that one is launched without the attribute
+// (PairLaunch::lead).
 // No pass triggers its dependents itself (griddepcontrol.launch_dependents): a
 // trigger at the start of the blocks let the next pass's blocks pile up on the
 // few SMs with free slots, where they waited and then ran, while the other SMs
@@ -1672,7 +1676,7 @@ void launch_plane_as(const PairLaunch& L, const Batch& b, int pass, cudaStream_t
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     } else {
-      launch_pdl(!L.no_pdl, kern, grid, blk, smem, st, P);
+      launch_pdl(!L.no_pdl && !(pass == 0 && L.lead), kern, grid, blk, smem, st, P);
     }
   };
   if constexpr (SPLIT) {
