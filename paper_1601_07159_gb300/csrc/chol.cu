@@ -56,26 +56,11 @@ __global__ void neg_copy_kernel(const double2* __restrict__ M, long long count, 
   if (i < count) A[i] = make_double2(-M[i].x, -M[i].y);
 }
 
-// r ~ 1 / d and y ~ 1 / sqrt(d) for a positive finite d: the hardware's 20-bit
-// approximations (they flush subnormal numbers) and one cubic step, e = 1 - d r: r (1 + e + e^2), e = 1 - d y^2:
-// y (1 + e / 2 + 3 e^2 / 8) (2^-20 -> 2^-60, then rounding).
-// plain(): d positive with a binary exponent in [-930, 930], from the upper word (a
-// comparison of doubles costs as much as a multiply-add).
-__device__ __forceinline__ bool plain(double d) {
-  return (unsigned)(__double2hiint(d) - ((1023 - 930) << 20)) < (1860u << 20);
-}
-__device__ __forceinline__ double recip(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double e = fma(-d, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-__device__ __forceinline__ double recip_sqrt(double d) {
-  if (!plain(d)) return 1.0 / sqrt(d);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-d * y, y, 1.0);
-  return fma(y * e, fma(e, 0.375, 0.5), y);
+// d positive and finite, from its words (a comparison of doubles costs as much as a
+// multiply-add).
+__device__ __forceinline__ bool positive_finite(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d);
+  return hi < 0x7ff00000u && (hi | (unsigned)__double2loint(d)) != 0u;
 }
 
 // Factor and invert the diagonal block of panel p (nb <= NB). The block is padded to
@@ -90,14 +75,15 @@ __device__ __forceinline__ double recip_sqrt(double d) {
 // pivot: d_{j+1} = a_{j+1,j+1} - |a_{j+1,j}|^2 / d_j and its reciprocal, while the
 // others do step j (with the pivot taken from its element's thread and the inverse
 // formed afterwards, by recursive doubling, the kernel took 22.4 us; 10.7 so).
-// At the end L_ik = a_ik / sqrt(d_k), and row i of X is divided by sqrt(d_i).
+// At the end L_ik = a_ik / sqrt(d_k), and row i of X is divided by sqrt(d_i). Reciprocals
+// and roots are CUDA's division and square root, correctly rounded.
 constexpr int kTri = NB * (NB + 1) / 2;             // lower-triangle elements
 constexpr int PIV = (kTri + 31) / 32;               // the pivot's warp, after the elements'
 __global__ void __launch_bounds__((PIV + 1) * 32)
 diag_kernel(double2* __restrict__ A, double2* __restrict__ X, int n, int p0, int nb, int* status) {
   __shared__ double2 col[2][NB], row[2][NB];        // a_ij (i > j) and x_jc (c <= j) of step j
   __shared__ double dg[2], rj[2];                   // a_{j+1,j+1} before step j, 1 / d_j
-  __shared__ double dd[NB], y[NB];                  // d_j, 1 / sqrt(d_j)
+  __shared__ double dd[NB], y[NB];                  // d_j, then its root; 1 / sqrt(d_j)
   __shared__ int s_fail, s_piv;
   const int tid = threadIdx.x, w = tid >> 5;
   if (status[0] != 0) return;
@@ -115,9 +101,7 @@ diag_kernel(double2* __restrict__ A, double2* __restrict__ X, int n, int p0, int
   }
   auto pivot = [&](int j, double d) {               // lane 0 of warp PIV: check d_j, keep it and its reciprocal
     dd[j] = d;
-    if (plain(d)) {
-      rj[j & 1] = recip(d);
-    } else if (isfinite(d) && d > 0.0) {
+    if (positive_finite(d)) {
       rj[j & 1] = 1.0 / d;
     } else {
       s_fail = isfinite(d) ? -2 : -3;
@@ -162,13 +146,16 @@ diag_kernel(double2* __restrict__ A, double2* __restrict__ X, int n, int p0, int
     }
     __syncthreads();
   }
-  if (tid < NB) y[tid] = recip_sqrt(dd[tid]);
+  if (tid < NB) {
+    dd[tid] = sqrt(dd[tid]);
+    y[tid] = 1.0 / dd[tid];
+  }
   __syncthreads();
   if (!elem || i >= nb) return;
   const double yi = y[i], yk = y[k];
   const long long o = (long long)(p0 + i) * n + p0 + k;
   if (i == k) {
-    A[o] = make_double2(dd[i] * yi, 0.0);
+    A[o] = make_double2(dd[i], 0.0);
     X[o] = make_double2(yi, 0.0);
   } else {
     A[o] = make_double2(l.x * yk, l.y * yk);
