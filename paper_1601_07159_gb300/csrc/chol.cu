@@ -74,7 +74,9 @@ __device__ __forceinline__ bool positive_finite(double d) {
 // the step before (two buffers, one barrier a step). Warp PIV works ahead on the
 // pivot: d_{j+1} = a_{j+1,j+1} - |a_{j+1,j}|^2 / d_j and its reciprocal, while the
 // others do step j (with the pivot taken from its element's thread and the inverse
-// formed afterwards, by recursive doubling, the kernel took 22.4 us; 10.7 so).
+// formed afterwards, by recursive doubling, the kernel took 22.4 us; 10.7 so). What it
+// leaves for a step (the pivot's reciprocal and verdict) lies in the word of that
+// step's parity, which no thread reads before the barrier.
 // At the end L_ik = a_ik / sqrt(d_k), and row i of X is divided by sqrt(d_i). Reciprocals
 // and roots are CUDA's division and square root, correctly rounded.
 constexpr int kTri = NB * (NB + 1) / 2;             // lower-triangle elements
@@ -84,7 +86,7 @@ diag_kernel(double2* __restrict__ A, double2* __restrict__ X, int n, int p0, int
   __shared__ double2 col[2][NB], row[2][NB];        // a_ij (i > j) and x_jc (c <= j) of step j
   __shared__ double dg[2], rj[2];                   // a_{j+1,j+1} before step j, 1 / d_j
   __shared__ double dd[NB], y[NB];                  // d_j, then its root; 1 / sqrt(d_j)
-  __shared__ int s_fail, s_piv;
+  __shared__ int fail[2];                           // status code of pivot j at j & 1 (0: good)
   const int tid = threadIdx.x, w = tid >> 5;
   if (status[0] != 0) return;
   // element (i, k) of thread tid: rows in decreasing order, so that the elements of a
@@ -100,31 +102,26 @@ diag_kernel(double2* __restrict__ A, double2* __restrict__ X, int n, int p0, int
     if (i == 1 && k == 1) dg[0] = v.x;
   }
   auto pivot = [&](int j, double d) {               // lane 0 of warp PIV: check d_j, keep it and its reciprocal
+    const bool ok = positive_finite(d);
     dd[j] = d;
-    if (positive_finite(d)) {
-      rj[j & 1] = 1.0 / d;
-    } else {
-      s_fail = isfinite(d) ? -2 : -3;
-      s_piv = j;
-    }
+    fail[j & 1] = ok ? 0 : isfinite(d) ? -2 : -3;
+    if (ok) rj[j & 1] = 1.0 / d;
   };
-  if (tid == 0) {
-    s_fail = 0;
-    row[0][0] = make_double2(1.0, 0.0);
-  }
+  if (tid == 0) row[0][0] = make_double2(1.0, 0.0);
   __syncthreads();
   if (tid == PIV * 32) pivot(0, col[0][0].x);
   __syncthreads();
   double2 l = v;                                    // a_ik once it is final
   for (int j = 0; j < NB; ++j) {
-    if (s_fail) {                                   // uniform: read after a barrier
+    const int c = j & 1;
+    // pivot j's word: written in the step before; this step writes the other one
+    if (fail[c]) {
       if (tid == 0) {
-        status[0] = s_fail;
-        status[1] = p0 + s_piv + 1;
+        status[0] = fail[c];
+        status[1] = p0 + j + 1;
       }
       return;
     }
-    const int c = j & 1;
     const double r = rj[c];
     if (w == PIV) {
       if (tid == PIV * 32 && j + 1 < NB) {
