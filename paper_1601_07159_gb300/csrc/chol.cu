@@ -63,6 +63,14 @@ __device__ __forceinline__ bool positive_finite(double d) {
   return hi < 0x7ff00000u && (hi | (unsigned)__double2loint(d)) != 0u;
 }
 
+// a - |u|^2 r, with one dependent operation after r where |u|^2 cannot leave the range of
+// doubles (the larger component's exponent in [-480, 480)), else by products with u r.
+__device__ __forceinline__ double minus_abs2(double a, double2 u, double r) {
+  const int e = max(__double2hiint(u.x) & 0x7fffffff, __double2hiint(u.y) & 0x7fffffff) >> 20;
+  if ((unsigned)(e - (1023 - 480)) < 960u) return fma(-fma(u.x, u.x, u.y * u.y), r, a);
+  return fma(-u.y * r, u.y, fma(-u.x * r, u.x, a));
+}
+
 // Factor and invert the diagonal block of panel p (nb <= NB). The block is padded to
 // NB with the identity, so every loop runs NB uniform steps.
 // Elimination on unscaled columns, -M = L' D L'^*: step j subtracts
@@ -126,7 +134,7 @@ diag_kernel(double2* __restrict__ A, double2* __restrict__ X, int n, int p0, int
     if (w == PIV) {
       if (tid == PIV * 32 && j + 1 < NB) {
         const double2 u = col[c][j + 1];
-        pivot(j + 1, fma(-fma(u.x, u.x, u.y * u.y), r, dg[c]));
+        pivot(j + 1, minus_abs2(dg[c], u, r));
       }
     } else if (elem && i > j) {
       if (k == j) {                                 // a_ij is final: on to x_ij, which starts at zero
