@@ -952,7 +952,7 @@ ace_status ace_plan_create(const ace_desc* d, ace_plan** out) {
     launch_one(p, prep, none, nullptr);
     prepare_cholesky(N);
     if (p->tc) tc_gemm_prepare();
-    if (p->apply16) apply_tc_prepare();
+    if (p->apply16) p->apply16 = apply_tc_prepare();   // else the TF32 products
     if (p->xi == 1) xi_oz_prepare();
     if (p->engine) {
       if (p->f64) engine_prepare_f64(p->nx, p->einfo);
@@ -1428,9 +1428,11 @@ ace_status ace_apply(ace_plan* p, const void* Xi, const void* Psi, int nb, void*
   // C = dV Xi^* Psi, Y = -Xi C (Eq. ACE)
   if (p->apply16 && apply_tc_faster(p->ng, N, nb)) {
     const int k = launch_apply_tc(Xi, N, Psi, nb, p->ld, p->ng, p->dv, Y, ws, Wl.total, p->status, st);
-    if (k == 0) return fail(ACE_ERR_CUDA, "tensor map encoding failed");
-    p->launches += k;
-    return cuda_check("ace_apply");
+    if (k > 0) {
+      p->launches += k;
+      return cuda_check("ace_apply");
+    }
+    // no tensor map for these vectors (2^40 bytes or more apart): the TF32 products
   }
   const int splits = gram_parts(p, N, nb);
   if (p->tc) launch_gram_tc(Xi, N, Psi, nb, p->ld, p->ng, Wl.part, splits, p->status, st, p->bf16);

@@ -1,0 +1,53 @@
+"""The apply of complex FP32 plans on vectors at the limits of what its FP16 operand
+pairs and tensor maps take, on a grid that runs them (2^16 points or more): against
+the oracle.
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+GRID = (40, 48, 36)
+DV = 0.43 ** 3
+TOL = 1e-5    # per band, as in the other FP32 apply tests
+
+
+@pytest.fixture(scope="module")
+def ace():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1601_07159_gb300 import build_lib
+    build_lib.build()
+    from paper_1601_07159_gb300 import ace as mod
+    return mod
+
+
+def _plan(ace, nocc, **kw):
+    return ace.Plan(GRID, tuple(0.43 * g for g in GRID), nocc, dtype="c64", **kw)
+
+
+def _random(rng, n):
+    return rng.standard_normal((n, *GRID[::-1], 2), dtype=np.float32).view(np.complex64)[..., 0]
+
+
+def _apply(plan, xi, psi):
+    y = plan.apply(torch.from_numpy(xi).cuda(), torch.from_numpy(psi).cuda(), out=torch.empty(psi.shape, dtype=torch.complex64, device="cuda"))
+    assert plan.status() == (0, 0)
+    return y.cpu().numpy().astype(np.complex128)
+
+
+def _want(xi, psi):
+    return oracle.ace_apply(xi.astype(np.complex128), psi.astype(np.complex128), DV)
+
+
+@pytest.mark.parametrize("ld", [1 << 36, 1 << 37, 1 << 40])
+def test_strides_beyond_a_tensor_map(ace, ld):
+    """One orbital, one band: the distance to a next vector is never used, so any is
+    taken. A tensor map's is below 2^40 bytes (2^37 elements)."""
+    rng = np.random.default_rng(1)
+    xi, psi = _random(rng, 1), _random(rng, 1)
+    got, want = _apply(_plan(ace, 1, ld=ld), xi, psi), _want(xi, psi)
+    assert np.linalg.norm(got - want) < TOL * np.linalg.norm(want)
