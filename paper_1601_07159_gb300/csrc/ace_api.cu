@@ -300,6 +300,10 @@ struct WsLayout {
 int gram_parts(const ace_plan* p, int na, int nb) {
   return p->tc ? gram_tc_splits(p->ng, na, nb) : gram_splits(p->f64, p->ng, na, nb);
 }
+// Doubles that hold them.
+size_t part_doubles(const ace_plan* p, int na, int nb) {
+  return 2 * (p->tc ? (size_t)gram_parts(p, na, nb) * na * nb : gram_part_entries(p->f64, p->ng, na, nb));
+}
 
 // Upper bound on the batches of the one-sided schedule for n_b vectors.
 long long rect_batch_bound(const ace_plan* p, int nb) {
@@ -317,7 +321,6 @@ WsLayout layout(const ace_plan* p, int op, int nb, char* base) {
   size_t off = 0;
   auto take = [&](size_t bytes) { char* r = base ? base + off : nullptr; off += align256(bytes); return r; };
   const int N = p->d.n_occ;
-  const int splits = op == ACE_OP_BUILD_OVERSAMPLED ? gram_parts(p, nb, nb) : gram_parts(p, N, op == ACE_OP_APPLY ? nb : N);
   if (op == ACE_OP_EXCHANGE_APPLY || op == ACE_OP_BUILD || op == ACE_OP_ENERGY_GRAD || op == ACE_OP_BUILD_OVERSAMPLED ||
       op == ACE_OP_POISSON || op == ACE_OP_ENERGY_GRAD_STORE) {
     L.S = take((size_t)p->lanes * lane_bytes(p));
@@ -327,7 +330,7 @@ WsLayout layout(const ace_plan* p, int op, int nb, char* base) {
     L.ctr = take(engine_ctr_bytes(nbat));
   }
   if (op == ACE_OP_BUILD_OVERSAMPLED) {
-    const size_t pd = (size_t)splits * nb * nb * 2;
+    const size_t pd = part_doubles(p, nb, nb);
     L.part = (double*)take((pd > diag_dot_part_doubles(nb) ? pd : diag_dot_part_doubles(nb)) * sizeof(double));
     L.Wtmp = take((size_t)nb * p->ld * p->vsize);
     L.Cm = (double*)take((size_t)nb * nb * 2 * sizeof(double));
@@ -343,13 +346,13 @@ WsLayout layout(const ace_plan* p, int op, int nb, char* base) {
     L.store = take((size_t)slots * slot_bytes(p));
   }
   if (op == ACE_OP_BUILD) {
-    const size_t pd = (size_t)splits * N * N * 2;
+    const size_t pd = part_doubles(p, N, N);
     L.part = (double*)take((pd > diag_dot_part_doubles(N) ? pd : diag_dot_part_doubles(N)) * sizeof(double));
     L.Wtmp = take((size_t)N * p->ld * p->vsize);
     if (p->xi == 1) L.xis = take(xi_oz_scratch_bytes(p->ng, N, N, false));
   }
   if (op == ACE_OP_APPLY) {
-    L.part = (double*)take((size_t)splits * N * nb * 2 * sizeof(double));
+    L.part = (double*)take(part_doubles(p, N, nb) * sizeof(double));
     L.Cm = (double*)take((size_t)N * nb * 2 * sizeof(double));
     // a few bands or orbitals: the FP16 products' padded right operand is the larger
     if (p->apply16 && nb > 0 && off < apply_tc_least_bytes(p->ng, N, nb)) off = apply_tc_least_bytes(p->ng, N, nb);

@@ -117,6 +117,7 @@ int energy_blocks(int nx, int ny, int nz, int npairs);
 void launch_gram(bool f64, bool real_in, const void* A, int na, const void* B, int nb, long long ld,
                  long long ng, double* part, int splits, cudaStream_t st);
 int gram_splits(bool f64, long long ng, int na, int nb);
+size_t gram_part_entries(bool f64, long long ng, int na, int nb);   // complex FP64 entries of `part`
 int launch_gram_reduce(const double* part, int splits, int na, int nb, double scale, bool hermitize,
                        bool real_out, double* out, double* out_trace_half, cudaStream_t st);
 // upper: C is upper triangular (L^{-*}); the FP64 product skips its zeros.

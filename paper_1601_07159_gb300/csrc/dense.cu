@@ -8,6 +8,7 @@
 // Arrays of vectors are orbital-major [count][N_g] (x fastest); small matrices
 // are row-major FP64 (complex interleaved). The GEMMs run on CUDA cores in the
 // vectors' precision with a deterministic split-K reduction in FP64.
+#include <algorithm>
 #include <cmath>
 
 #include "ace_internal.h"
@@ -148,22 +149,41 @@ gram64_kernel(const void* __restrict__ A, int na, const void* __restrict__ B, in
   }
 }
 
+namespace {
+constexpr long long kGramBlocks64 = 4 * 152;   // FP64: four blocks per SM
+constexpr long long kMaxGramSplits = 256;
+long long gram_tiles(bool f64, int na, int nb) {
+  const int edge = f64 ? GT64 : GT;
+  return (long long)((na + edge - 1) / edge) * ((nb + edge - 1) / edge);
+}
+}  // namespace
+
 int gram_splits(bool f64, long long ng, int na, int nb) {
   // ~1k-point chunks keep the partial sums short; small matrices on small grids
   // take shorter chunks so that the launch still covers one wave of SMs (FP64:
   // four blocks per SM, whose tiles are small)
   long long s = (ng + 1023) / 1024;
-  const int edge = f64 ? GT64 : GT;
-  const long long tiles = (long long)((na + edge - 1) / edge) * ((nb + edge - 1) / edge);
-  const long long blocks = f64 ? 4 * 152 : 152;
+  const long long tiles = gram_tiles(f64, na, nb);
+  const long long blocks = f64 ? kGramBlocks64 : 152;
   const long long wave = tiles > 0 ? (blocks + tiles - 1) / tiles : 1;
   const long long stage = f64 ? GK64 : GK;
   const long long max_s = (ng + stage - 1) / stage;   // at least one K stage per split
   if (s < wave) s = wave;
   if (s > max_s) s = max_s;
-  if (s > 256) s = 256;
+  if (s > kMaxGramSplits) s = kMaxGramSplits;
   if (s < 1) s = 1;
   return (int)s;
+}
+
+// Entries to hold the partial matrices: for FP64 a bound on gram_splits() na nb that
+// never falls as na or nb grows (a workspace sized for the widest call serves every
+// narrower one; the splits of 8 x 8 tiles halve as tiles double, so the product itself
+// does). With na nb <= 64 tiles, na nb ceil(blocks / tiles) <= 64 (blocks + tiles).
+size_t gram_part_entries(bool f64, long long ng, int na, int nb) {
+  if (!f64) return (size_t)gram_splits(f64, ng, na, nb) * na * nb;
+  const long long points = std::min((ng + 1023) / 1024, kMaxGramSplits);
+  const long long wave = std::min(kMaxGramSplits * na * nb, 64 * (kGramBlocks64 + gram_tiles(f64, na, nb)));
+  return (size_t)std::max(points * na * nb, wave);
 }
 
 void launch_gram(bool f64, bool real_in, const void* A, int na, const void* B, int nb, long long ld,
