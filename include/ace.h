@@ -127,8 +127,8 @@ typedef struct {
   int tile;          /* orbitals per pair tile, 1..8 (0 = default 8) */
   int lanes;         /* concurrent batch streams inside one call with
                         ACE_FLAG_NO_OVERLAP, 1..8 (0 = default 2; without the flag
-                        1 for C64, at least 2 for FP64); the pair scratch is
-                        lanes * max_pairs slots */
+                        always 1 for C64 plans that replay graphs, at least 2 for
+                        FP64); the pair scratch is lanes * max_pairs slots */
   int flags;         /* ACE_FLAG_* */
 } ace_desc;
 

@@ -866,7 +866,7 @@ ace_status ace_plan_create(const ace_desc* d, ace_plan** out) {
   p->xi = xi_slices ? 1 : (d->prec == ACE_PREC_XI_FP64_SIMT ? 2 : 0);
   p->overlap = p->graphs && !p->engine && !(d->flags & ACE_FLAG_NO_OVERLAP);
   if (p->overlap && p->f64 && p->lanes < 2) p->lanes = 2;   // two scratch buffers
-  if (p->overlap && !p->f64 && !d->lanes) p->lanes = 1;     // one
+  if (p->overlap && !p->f64) p->lanes = 1;                  // one chain in one buffer, whatever was asked for
   p->radix = (!p->f64 && (d->flags & ACE_FLAG_RADIX_ODD_FIRST)) ? 1 : 0;
   const size_t slot = (size_t)p->ng * p->csize;
   const int tt = p->tile * p->tile;

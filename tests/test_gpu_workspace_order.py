@@ -39,3 +39,15 @@ def test_narrower_block_in_a_wider_workspace(ace):
     p = lambda t: ctypes.c_void_p(t.data_ptr())   # noqa: E731
     assert ace.lib().ace_apply(plan._h, p(xi), p(psi), 32, p(y), p(ws), ws.numel(), None) == ace.ACE_OK
     assert torch.equal(y, plan.apply(xi, psi))
+
+
+@pytest.mark.parametrize("lanes", [2, 3])
+def test_one_chain_takes_one_buffer(ace, lanes):
+    """C64 plans run their passes as one chain in one scratch buffer; a tuned schedule's
+    lanes (which belong to the form without overlap) add none."""
+    for op in (ace.OP_BUILD, ace.OP_ENERGY_GRAD, ace.OP_EXCHANGE_APPLY):
+        plans = [ace.Plan(24, 10.0, 20, dtype="c64", max_pairs=64, lanes=k) for k in (0, lanes)]
+        assert plans[0].workspace_size(op, 5) == plans[1].workspace_size(op, 5)
+    spread = ace.Plan(24, 10.0, 20, dtype="c64", max_pairs=64, lanes=lanes, overlap=False)
+    assert spread.workspace_size(ace.OP_BUILD) > plans[0].workspace_size(ace.OP_BUILD)
+    assert spread.effective_schedule()["lanes"] == lanes
