@@ -79,10 +79,12 @@ typedef enum {
  *    FP32 operand split into two TF32 terms, three products (FP32 accuracy).
  *  ACE_PREC_XI_FP64 (the C64 default, ACE_PREC_DEFAULT): M as SPLIT_TF32. The
  *    apply's products, from 2^16 grid points or 7 2^18 values in Xi and Psi together
- *    on, run on the FP16 tensor cores: every vector scaled by a power of two, every value split into two
- *    FP16 terms, three products (FP32 accuracy: an operand's error is below 2^-22 of
- *    itself, or 2^-40 of its vector's largest value if that is more); smaller
- *    calls as SPLIT_TF32. Xi = W L^{-*} is computed to FP64 accuracy from the FP32 W and the
+ *    on, run on the FP16 tensor cores: operands scaled by powers of two, every value
+ *    split into two FP16 terms, three products (FP32 accuracy: an operand's error is
+ *    below 2^-22 of itself, or 2^-40 of the largest value that shares its scale if that
+ *    is more: in C = dV Xi^* Psi the largest of its vector; in Y = -Xi C the largest of
+ *    any Xi_k at the same point, and of any C_kb of the same band); smaller calls as
+ *    SPLIT_TF32. Xi = W L^{-*} is computed to FP64 accuracy from the FP32 W and the
  *    FP64 L^{-*} on the FP16 tensor cores (error-free 8-bit integer slices of
  *    both operands, exact integer products, exact accumulation) and rounded
  *    once to FP32: before that rounding the error of Xi_b(g) is below about

@@ -1,11 +1,16 @@
 // Tensor-core products of the ACE apply (Eq. ACE: C = dV Xi^* psi, Y = -Xi C) for
 // complex FP32 vectors, on tcgen05 kind::f16 with FP16 operand pairs.
 //
-// FP32 accuracy from FP16 operands: every vector is scaled by a power of two that
-// puts its largest component in [2^14, 2^15), and a scaled value x is split x =
-// hi + lo, hi = fp16(x), lo = fp16(x - hi) (round to nearest). hi and lo carry 22
-// to 23 bits of every value down to 2^-18 of the vector's largest (lo is then a
-// normal FP16 number) and below that an absolute error of 2^-40 of the largest.
+// FP32 accuracy from FP16 operands: a row or column of an operand is scaled by a power
+// of two that puts its largest component in [2^14, 2^15), and a scaled value x is
+// split x = hi + lo, hi = fp16(x), lo = fp16(x - hi) (round to nearest; the splitting
+// of Markidis et al., "NVIDIA Tensor Core Programmability, Performance & Precision",
+// 2018, with both parts scaled). hi and lo carry 22 to 23 bits of every value down to
+// 2^-18 of the row's largest (lo is then a normal FP16 number) and below that an absolute
+// error of 2^-40 of the largest. So what shares a scale matters: the gram product's
+// rows and columns are vectors; the outer product's rows are points (the largest value
+// of any orbital there), so that V_ACE psi keeps its relative accuracy where every
+// orbital is small, as in vacuum, and its columns are the bands' coefficients.
 // Three products hi hi + hi lo + lo hi are kept; the dropped lo lo is below
 // 2^-24. (The TF32 split of tc_gemm.cu truncates both parts and drops 2^-20.) A
 // kind::f16 MMA does twice the work of a kind::tf32 one per cycle on half the
@@ -227,35 +232,52 @@ template <int TN> __device__ __forceinline__ void teardown(uint32_t tmem) {
   if (threadIdx.x < 32) tc::tmem_dealloc_warp(tmem, Tile<TN>::TMEM_COLS);
 }
 
-// Largest |component| of each vector (as float bits, which order like the values;
-// NaN is skipped): vectors [0, na) of A into mx[0 .. na), of B into mx[na ..).
+// Largest |component| (as float bits, which order like the values; NaN is skipped) of
+// each vector, mx[0 .. na) for A and mx[na ..) for B, and of each point over the vectors
+// of A, pt[g]. Grid: (ya parts of `per` vectors of A and then those of B, 512-point
+// segments). A warp takes a segment of one vector at a time, eight 16-byte loads in flight a
+// thread, and keeps the maxima of its points in registers; one sweep of the vectors,
+// bound by memory.
+constexpr int SEG = 512;
 __global__ void __launch_bounds__(256)
-vec_max_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B, long long ld, long long ng,
-               unsigned* __restrict__ mx) {
-  const int v = blockIdx.x;
-  const float4* x = reinterpret_cast<const float4*>(v < na ? A + (long long)v * ld : B + (long long)(v - na) * ld);
-  const long long n = ng / 2, step = (long long)gridDim.y * blockDim.x;   // N_g is even on every grid
-  float m = 0.f;
-  long long i = (long long)blockIdx.y * blockDim.x + threadIdx.x;
-  for (; i + 3 * step < n; i += 4 * step) {
-    float4 t[4];
+maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B, int nb, long long ld, long long ng,
+              int per, int ya, unsigned* __restrict__ mx, unsigned* __restrict__ pt) {
+  const bool first = (int)blockIdx.x < ya;               // a part of A
+  const int count = first ? na : nb, v0 = ((int)blockIdx.x - (first ? 0 : ya)) * per;
+  const int v1 = v0 + per < count ? v0 + per : count;
+  const float2* X = first ? A : B;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long n = ng / 2, i0 = (long long)blockIdx.y * (SEG / 2);   // float4 units: N_g is even on every grid
+  float2 p[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) t[u] = x[i + u * step];
+  for (int u = 0; u < 8; ++u) p[u] = make_float2(0.f, 0.f);
+  for (int v = v0 + w; v < v1; v += 8) {
+    const float4* x = reinterpret_cast<const float4*>(X + (long long)v * ld) + i0 + lane;
+    float4 t[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      m = fmaxf(m, fmaxf(fmaxf(fabsf(t[u].x), fabsf(t[u].y)), fmaxf(fabsf(t[u].z), fabsf(t[u].w))));
+    for (int u = 0; u < 8; ++u) t[u] = i0 + lane + 32 * u < n ? x[32 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float m = 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const float a = fmaxf(fabsf(t[u].x), fabsf(t[u].y)), b = fmaxf(fabsf(t[u].z), fabsf(t[u].w));
+      p[u] = make_float2(fmaxf(p[u].x, a), fmaxf(p[u].y, b));
+      m = fmaxf(m, fmaxf(a, b));
+    }
+    const unsigned r = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if (lane == 0) atomicMax(mx + (first ? v : na + v), r);
   }
-  for (; i < n; i += step) {
-    const float4 t = x[i];
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(t.x), fabsf(t.y)), fmaxf(fabsf(t.z), fabsf(t.w))));
-  }
-  unsigned b = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-  __shared__ unsigned red[8];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = b;
+  if (!first) return;
+  __shared__ float2 red[8][SEG / 2];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) red[w][lane + 32 * u] = p[u];
   __syncthreads();
-  if (threadIdx.x < 32) {
-    b = __reduce_max_sync(0xffffffffu, threadIdx.x < 8 ? red[threadIdx.x] : 0u);
-    if (threadIdx.x == 0) atomicMax(mx + v, b);
+  const int i = threadIdx.x;
+  float2 q = red[0][i];
+#pragma unroll
+  for (int k = 1; k < 8; ++k) q = make_float2(fmaxf(q.x, red[k][i].x), fmaxf(q.y, red[k][i].y));
+  if (i0 + i < n) {
+    atomicMax(pt + 2 * (i0 + i), __float_as_uint(q.x));
+    atomicMax(pt + 2 * (i0 + i) + 1, __float_as_uint(q.y));
   }
 }
 
@@ -464,27 +486,27 @@ gram16_reduce_kernel(const float2* __restrict__ part, int splits, long long tota
 }
 
 // The outer product's right operand. With Xi_k = 2^-e_k X_k and psi_b = 2^-e_b P_b (X, P
-// the scaled vectors, C their products), Y_b = -sum_k X_k (2^-2e_k C_kb) 2^-e_b: column b of
-// 2^-2e_k C_kb, scaled by its own power of two 2^f to [2^14, 2^15), is split and written in the
+// the scaled vectors, C their products), Y_b = -sum_k Xi_k (2^-e_k C_kb) 2^-e_b: column b of
+// 2^-e_k C_kb, scaled by its own power of two 2^f to [2^14, 2^15), is split and written in the
 // stage layout of (column tile bt, chunk c): [bt][c] holds B_hi, B_lo tiles of TN rows
 // x 32 K. Eight columns per block (padding columns and rows are written as zeros).
-// colscale[b]: two factors of 2^-(f + e_b), whose exponent can leave FP32's range.
+// colexp[b] = -(f + e_b): the exponent that takes column b's products back.
 template <int TN>
 __global__ void __launch_bounds__(256)
 c_split_kernel(const float2* __restrict__ C, int nk, int nb, int nch, const unsigned* __restrict__ mx,
-               unsigned char* __restrict__ Bs, float2* __restrict__ colscale) {
+               unsigned char* __restrict__ Bs, int* __restrict__ colexp) {
   using T = Tile<TN>;
   __shared__ int red[32][8];
   const int j8 = threadIdx.x & 7, kl = threadIdx.x >> 3;
   const int col = blockIdx.x * 8 + j8, bt = col / T::BB, j = col - bt * T::BB;
-  // the largest biased exponent of 2^-2e_k max(|re|, |im|)
+  // the largest biased exponent of 2^-e_k max(|re|, |im|)
   constexpr int kNone = -100000;
   int m = kNone;
   if (col < nb)
     for (int k = kl; k < nk; k += 32) {
       const float2 c = C[(long long)k * nb + col];
       const int e = (int)((max(__float_as_uint(c.x) & 0x7fffffffu, __float_as_uint(c.y) & 0x7fffffffu)) >> 23);
-      if (e != 0) m = max(m, e - 2 * scale_exp(mx[k]));
+      if (e != 0) m = max(m, e - scale_exp(mx[k]));
     }
   red[kl][j8] = m;
   __syncthreads();
@@ -493,15 +515,12 @@ c_split_kernel(const float2* __restrict__ C, int nk, int nb, int nch, const unsi
     __syncthreads();
   }
   const int f = red[0][j8] == kNone ? 0 : 141 - red[0][j8];
-  if (kl == 0 && col < nb) {
-    const int g = -(f + scale_exp(mx[nk + col])), h = max(-126, min(126, g));
-    colscale[col] = make_float2(exp2i(h), ldexpf(1.f, g - h));
-  }
+  if (kl == 0 && col < nb) colexp[col] = -(f + scale_exp(mx[nk + col]));
   for (int k = kl; k < nch * 16; k += 32) {
     float2 x = make_float2(0.f, 0.f);
     if (col < nb && k < nk) {
       const float2 c = C[(long long)k * nb + col];
-      const int g = f - 2 * scale_exp(mx[k]);
+      const int g = f - scale_exp(mx[k]);
       x = make_float2(ldexpf(c.x, g), ldexpf(c.y, g));
     }
     const __half2 hi = __float22half2_rn(x);
@@ -526,11 +545,12 @@ c_split_kernel(const float2* __restrict__ C, int nk, int nb, int nch, const unsi
 // stores. A chunk's 16 orbital rows (1 KB each, one TMA box) and its right operand (one
 // bulk copy) arrive on one mbarrier, issued by one thread RING - 2 chunks ahead: its slots are
 // those of chunk n - 2, whose MMAs have just ended. Thread t owns point t % 128 and
-// orbitals 4 (t / 128) .. + 3 of each chunk.
+// orbitals 4 (t / 128) .. + 3 of each chunk. Row g is scaled by the power of two of the
+// point's largest value, pt[g], which the stores take back with the column's.
 template <int TN>
 __global__ void __launch_bounds__(THREADS, 1)
-outer16_kernel(const __grid_constant__ CUtensorMap A, int nk, int nb, long long ld, long long ng, float alpha,
-               const unsigned* __restrict__ mx, const unsigned char* __restrict__ Bs, const float2* __restrict__ colscale,
+outer16_kernel(const __grid_constant__ CUtensorMap A, int nb, long long ld, long long ng, float alpha,
+               const unsigned* __restrict__ pt, const unsigned char* __restrict__ Bs, const int* __restrict__ colexp,
                int nch, float2* __restrict__ Out, int* status) {
   using T = Tile<TN>;
   constexpr int BB = T::BB, NH = T::NH, R = T::O_RING;
@@ -538,7 +558,7 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nk, int nb, long long 
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* bring = base + 2 * T::O_STAGE;
   unsigned char* ring = bring + R * T::O_B;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ring + R * T::O_RAW);   // [0, 2): MMAs of a stage; [2, 6): a chunk landed
+  uint64_t* bar = reinterpret_cast<uint64_t*>(ring + R * T::O_RAW);   // [0, 2): MMAs of a stage; then R: a chunk landed
   __shared__ int s_fail;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   if (tid == 0) s_fail = 0;
@@ -575,12 +595,15 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nk, int nb, long long 
     const int bq = (tile - gt * nbt) * BB + NH * (w >> 2);
     if (g < ng) {
       float2* p = Out + (long long)bq * ld + g;
-      const float2* cs = colscale + bq;
+      const int* ce = colexp + bq;
+      const int er = 127 - scale_exp(__ldg(pt + g));
 #pragma unroll
       for (int j = 0; j < NH; ++j) {
         if (bq + j < nb) {
-          const float2 f = __ldg(cs + j);
-          *p = make_float2(f.y * (alpha * f.x * S.re[j]), f.y * (alpha * f.x * S.im[j]));
+          // the exponent in two factors: it can leave FP32's range where the value does not
+          const int e = er + __ldg(ce + j), e1 = max(1, min(254, e)), e2 = max(1, min(254, e - e1 + 127));
+          const float f = alpha * __uint_as_float((unsigned)e1 << 23), h = __uint_as_float((unsigned)e2 << 23);
+          *p = make_float2(h * (f * S.re[j]), h * (f * S.im[j]));
         }
         p += ld;
       }
@@ -607,13 +630,17 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nk, int nb, long long 
     }
   };
   const int o = tile_off(r, 8 * q);
-  float sc[4];
+  auto point_max = [&](int t) {                          // of this thread's point in tile t
+    const long long g = (long long)(t / nbt) * TM + r;
+    return t < ntiles && g < ng ? __ldg(pt + g) : 0u;
+  };
+  unsigned pnext = point_max(tile);
+  float sc = 0.f;
   for (int n = 0; n < total; ++n) {
     const int s = n & 1, slot = n % R;
-    const int k = c * (KC / 2) + 4 * q;
-    if (nch > 1 || n == 0) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) sc[i] = k + i < nk ? exp2i(scale_exp(__ldg(mx + k + i))) : 0.f;
+    if (c == 0) {
+      sc = exp2i(scale_exp(pnext));
+      pnext = point_max(tile + (int)gridDim.x);
     }
     if ((S.issued >> s) & 1u) finish(s);                 // the MMAs of chunk n - 2
     if (tid == 32) fetch();                              // into the slots that chunk n - 2 left
@@ -622,9 +649,7 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nk, int nb, long long 
     const float2* x = reinterpret_cast<const float2*>(ring + slot * T::O_RAW) + 4 * q * TM + r;
     uint32_t ah[4], al[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      split2(__fmul2_rn(x[i * TM], make_float2(sc[i], sc[i])), ah[i], al[i]);
-    }
+    for (int i = 0; i < 4; ++i) split2(__fmul2_rn(x[i * TM], make_float2(sc, sc)), ah[i], al[i]);
     unsigned char* st = base + s * T::O_STAGE + o;
     *reinterpret_cast<uint4*>(st) = make_uint4(ah[0], ah[1], ah[2], ah[3]);
     *reinterpret_cast<uint4*>(st + A_TILE) = make_uint4(al[0], al[1], al[2], al[3]);
@@ -727,13 +752,14 @@ int splits_for(long long ng, int na, int nb, long long cap) {
   return (int)best;
 }
 
-// Scratch layout: vector maxima, column scales, C, and the split sums, which the right
-// operand overwrites once they are reduced. The splits are those that fit `budget`
+// Scratch layout: vector and point maxima, column exponents, C, and the split sums, which
+// the right operand overwrites once they are reduced. The splits are those that fit `budget`
 // bytes (the plan's workspace is sized by the TF32 products, so that it does not depend on
 // a call's path); least = bytes for one.
 struct Scratch {
-  unsigned* mx;
-  float2* colscale;
+  unsigned* mx;      // vector maxima, then (at pt) point maxima
+  unsigned* pt;
+  int* colexp;
   unsigned char* Bs;
   float2* C;
   float2* part;
@@ -746,8 +772,9 @@ Scratch scratch(char* base, long long ng, int n, int nb, size_t budget) {
   auto take = [&](size_t bytes) { char* r = base ? base + off : nullptr; off += align256(bytes); return r; };
   const int bb = width(nb) / 2;
   const size_t nbt = (size_t)(nb + bb - 1) / bb, nch = (size_t)(n + 15) / 16;
-  s.mx = (unsigned*)take((size_t)(n + nb) * sizeof(unsigned));
-  s.colscale = (float2*)take((size_t)nb * sizeof(float2));
+  s.mx = (unsigned*)take(((size_t)(n + nb) + (size_t)ng) * sizeof(unsigned));
+  s.pt = s.mx + (n + nb);
+  s.colexp = (int*)take((size_t)nb * sizeof(int));
   s.C = (float2*)take((size_t)n * nb * sizeof(float2));
   s.part = (float2*)take(0);
   s.Bs = (unsigned char*)s.part;
@@ -812,11 +839,13 @@ int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld
   if (!encoder() || !vector_map(&xg, x, n, ld, ng, KC / 2, TM, true) ||
       !vector_map(&qg, psi, nb, ld, ng, KC / 2, width(nb) / 2, true) || !vector_map(&xo, x, n, ld, ng, TM, KC / 2, false))
     return 0;
-  cudaMemsetAsync(s.mx, 0, (size_t)(n + nb) * sizeof(unsigned), st);
-  // about 16 blocks per SM, at most one per 1024 points of a vector
-  long long per = (16 * 152 + n + nb - 1) / (n + nb), most = (ng / 2 + 1023) / 1024;
-  per = per < 1 ? 1 : per > most ? most : per;
-  vec_max_kernel<<<dim3(n + nb, (unsigned)per), 256, 0, st>>>(x, n, psi, ld, ng, s.mx);
+  cudaMemsetAsync(s.mx, 0, ((size_t)(n + nb) + (size_t)ng) * sizeof(unsigned), st);
+  // eight to 64 vectors per block (one to eight per warp), by what gives eight blocks per SM
+  const long long segs = (ng + SEG - 1) / SEG;
+  long long per = (segs * ((long long)n + nb) / (8 * 152) + 7) / 8 * 8;
+  per = per < 8 ? 8 : per > 64 ? 64 : per;
+  const int ya = (int)((n + per - 1) / per), yb = (int)((nb + per - 1) / per);
+  maxima_kernel<<<dim3(ya + yb, (unsigned)segs), 256, 0, st>>>(x, n, psi, nb, ld, ng, (int)per, ya, s.mx, s.pt);
   const int splits = s.splits, nch = (n + 15) / 16;
   long long chunk = (ng + splits - 1) / splits;
   chunk = (chunk + KC / 2 - 1) / (KC / 2) * (KC / 2);
@@ -830,10 +859,10 @@ int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld
     int ways = 8;
     while (ways > 1 && (ways > splits || total * ways > 152LL * 2048)) ways /= 2;
     gram16_reduce_kernel<<<(unsigned)((total * ways + 255) / 256), 256, 0, st>>>(s.part, splits, total, ways, dv, s.C);
-    c_split_kernel<TN><<<nbt * (T::BB / 8), 256, 0, st>>>(s.C, n, nb, nch, s.mx, s.Bs, s.colscale);
+    c_split_kernel<TN><<<nbt * (T::BB / 8), 256, 0, st>>>(s.C, n, nb, nch, s.mx, s.Bs, s.colexp);
     const long long ntiles = (long long)nbt * ((ng + TM - 1) / TM);
     outer16_kernel<TN><<<(unsigned)(ntiles < 152 ? ntiles : 152), THREADS, T::O_SMEM, st>>>(
-        xo, n, nb, ld, ng, -1.0f, s.mx, s.Bs, s.colscale, nch, static_cast<float2*>(Y), status);
+        xo, nb, ld, ng, -1.0f, s.pt, s.Bs, s.colexp, nch, static_cast<float2*>(Y), status);
   });
   return 5;
 }

@@ -51,3 +51,33 @@ def test_strides_beyond_a_tensor_map(ace, ld):
     xi, psi = _random(rng, 1), _random(rng, 1)
     got, want = _apply(_plan(ace, 1, ld=ld), xi, psi), _want(xi, psi)
     assert np.linalg.norm(got - want) < TOL * np.linalg.norm(want)
+
+
+def _near(rng, n, decades, axis_up=False):
+    """n vectors that share an envelope falling by `decades` along the last grid axis (rising
+    with axis_up), within a factor of two of it at every point: overlaps without
+    cancellation, so that an error per point shows."""
+    z = np.arange(GRID[2]) / (GRID[2] - 1)
+    env = 10.0 ** (-decades * (1 - z if axis_up else z))[None, :, None, None]
+    noise = rng.uniform(-0.5, 0.5, (n, *GRID[::-1])) + 1j * rng.uniform(-0.5, 0.5, (n, *GRID[::-1]))
+    return (env * (1.0 + noise)).astype(np.complex64)
+
+
+def _point_error(got, xi, psi):
+    """The largest error of a value over sum_k |Xi_k(r)| |C_kb|, its terms' size."""
+    x, p = xi.astype(np.complex128).reshape(len(xi), -1), psi.astype(np.complex128).reshape(len(psi), -1)
+    c = DV * (x.conj() @ p.T)
+    size = np.abs(c).T @ np.abs(x)
+    return float((np.abs(got.reshape(size.shape) + c.T @ x) / size).max())
+
+
+# The same bounds per value as per band: operands keep 22 bits of a value beside its
+# neighbours, the FP32 sums truncate at 2^-23 per group of 24 terms; 1e-5 as above.
+@pytest.mark.parametrize("nocc,nb", [(5, 3), (17, 40), (140, 100)])
+@pytest.mark.parametrize("prec", ["default", "split_tf32"])
+def test_accuracy_where_every_orbital_is_small(ace, prec, nocc, nb):
+    """Vacuum: every orbital decays by ten decades. The values there come as accurate,
+    relative to the orbitals there, as elsewhere."""
+    rng = np.random.default_rng(nocc)
+    xi, psi = _near(rng, nocc, 10.0), _near(rng, nb, 10.0)
+    assert _point_error(_apply(_plan(ace, nocc, prec=prec), xi, psi), xi, psi) < TOL
