@@ -354,8 +354,7 @@ WsLayout layout(const ace_plan* p, int op, int nb, char* base) {
   if (op == ACE_OP_APPLY) {
     L.part = (double*)take(part_doubles(p, N, nb) * sizeof(double));
     L.Cm = (double*)take((size_t)N * nb * 2 * sizeof(double));
-    // a few bands or orbitals: the FP16 products' padded right operand is the larger
-    if (p->apply16 && nb > 0 && off < apply_tc_least_bytes(p->ng, N, nb)) off = apply_tc_least_bytes(p->ng, N, nb);
+    if (p->apply16 && nb > 0) off = align256(apply_tc_bytes(p->ng, N, nb, off));
   }
   L.total = off;
   return L;

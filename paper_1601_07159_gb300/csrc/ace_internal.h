@@ -138,11 +138,11 @@ void launch_outer_tc(const void* A, int nk, const double* C, int nb, long long l
                      void* Out, void* c32, int* status, cudaStream_t st, bool bf16 = false);
 // The ACE apply Y = -Xi (dV Xi^* Psi) of n orbitals on nb vectors for complex FP32
 // (tc_apply.cu): FP16 operand pairs on the tensor cores, FP32 accuracy; ws of
-// `budget` bytes, at least apply_tc_least_bytes(). Returns the kernel count, 0 if
+// `budget` bytes, at least apply_tc_bytes(). Returns the kernel count, 0 if
 // nothing was launched.
 bool apply_tc_prepare();
 bool apply_tc_faster(long long ng, int n, int nb);   // than launch_gram_tc and launch_outer_tc
-size_t apply_tc_least_bytes(long long ng, int n, int nb);
+size_t apply_tc_bytes(long long ng, int n, int nb, size_t tf32);   // `tf32`: what the TF32 products take
 int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld, long long ng, double dv, void* Y,
                     void* ws, size_t budget, int* status, cudaStream_t st);
 // Xi = W L^{-*} with FP64 arithmetic from complex FP32 W (dense.cu): C upper

@@ -754,8 +754,8 @@ int splits_for(long long ng, int na, int nb, long long cap) {
 
 // Scratch layout: vector and point maxima, column exponents, C, and the split sums, which
 // the right operand overwrites once they are reduced. The splits are those that fit `budget`
-// bytes (the plan's workspace is sized by the TF32 products, so that it does not depend on
-// a call's path); least = bytes for one.
+// bytes: the plan's workspace holds what the TF32 products take, or `least` (one split)
+// if that is more, and the maxima of the points (`tables`) beside it.
 struct Scratch {
   unsigned* mx;      // vector maxima, then (at pt) point maxima
   unsigned* pt;
@@ -764,7 +764,7 @@ struct Scratch {
   float2* C;
   float2* part;
   int splits;
-  size_t least;
+  size_t least, tables;
 };
 Scratch scratch(char* base, long long ng, int n, int nb, size_t budget) {
   Scratch s{};
@@ -772,15 +772,16 @@ Scratch scratch(char* base, long long ng, int n, int nb, size_t budget) {
   auto take = [&](size_t bytes) { char* r = base ? base + off : nullptr; off += align256(bytes); return r; };
   const int bb = width(nb) / 2;
   const size_t nbt = (size_t)(nb + bb - 1) / bb, nch = (size_t)(n + 15) / 16;
-  s.mx = (unsigned*)take(((size_t)(n + nb) + (size_t)ng) * sizeof(unsigned));
-  s.pt = s.mx + (n + nb);
+  s.mx = (unsigned*)take((size_t)(n + nb) * sizeof(unsigned));
+  s.pt = (unsigned*)take((size_t)ng * sizeof(unsigned));   // behind mx: one memset clears both
+  s.tables = align256((size_t)ng * sizeof(unsigned));
   s.colexp = (int*)take((size_t)nb * sizeof(int));
   s.C = (float2*)take((size_t)n * nb * sizeof(float2));
   s.part = (float2*)take(0);
   s.Bs = (unsigned char*)s.part;
   const size_t one = (size_t)n * nb * sizeof(float2), bs = nbt * nch * (size_t)(2 * bb) * KC * 2 * 2;
-  s.least = off + align256(one > bs ? one : bs);
-  if (s.least <= budget) s.splits = splits_for(ng, n, nb, (long long)((budget - off) / one));
+  s.least = off - s.tables + align256(one > bs ? one : bs);
+  if (s.least + s.tables <= budget) s.splits = splits_for(ng, n, nb, (long long)((budget - off) / one));
   return s;
 }
 
@@ -828,7 +829,11 @@ bool apply_tc_faster(long long ng, int n, int nb) {
   return ng >= (1LL << 16) || ng * ((long long)n + nb) >= (7LL << 18);
 }
 
-size_t apply_tc_least_bytes(long long ng, int n, int nb) { return scratch(nullptr, ng, n, nb, 0).least; }
+size_t apply_tc_bytes(long long ng, int n, int nb, size_t tf32) {
+  const Scratch s = scratch(nullptr, ng, n, nb, 0);
+  const size_t b = tf32 > s.least ? tf32 : s.least;
+  return apply_tc_faster(ng, n, nb) ? b + s.tables : b;
+}
 
 int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld, long long ng, double dv, void* Y,
                     void* ws, size_t budget, int* status, cudaStream_t st) {
@@ -839,7 +844,7 @@ int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld
   if (!encoder() || !vector_map(&xg, x, n, ld, ng, KC / 2, TM, true) ||
       !vector_map(&qg, psi, nb, ld, ng, KC / 2, width(nb) / 2, true) || !vector_map(&xo, x, n, ld, ng, TM, KC / 2, false))
     return 0;
-  cudaMemsetAsync(s.mx, 0, ((size_t)(n + nb) + (size_t)ng) * sizeof(unsigned), st);
+  cudaMemsetAsync(s.mx, 0, (size_t)(reinterpret_cast<char*>(s.pt + ng) - reinterpret_cast<char*>(s.mx)), st);
   // eight to 64 vectors per block (one to eight per warp), by what gives eight blocks per SM
   const long long segs = (ng + SEG - 1) / SEG;
   long long per = (segs * ((long long)n + nb) / (8 * 152) + 7) / 8 * 8;
