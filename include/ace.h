@@ -81,9 +81,10 @@ typedef enum {
  *    apply's products, from 2^16 grid points or 7 2^18 values in Xi and Psi together
  *    on, run on the FP16 tensor cores: operands scaled by powers of two, every value
  *    split into two FP16 terms, three products (FP32 accuracy: an operand's error is
- *    below 2^-22 of itself, or 2^-40 of the largest value that shares its scale if that
- *    is more: in C = dV Xi^* Psi the largest of its vector; in Y = -Xi C the largest of
- *    any Xi_k at the same point, and of any C_kb of the same band); smaller calls as
+ *    below 2^-22 of itself or, if that is more, in C = dV Xi^* Psi 2^-36 of its vector's
+ *    largest value within a segment of 512 consecutive points, 2^-76 of its largest of
+ *    all, and in Y = -Xi C 2^-40 of the largest Xi_k at the same point and of the
+ *    largest C_kb of the same band; SPLIT_TF32 knows no such limits); smaller calls as
  *    SPLIT_TF32. Xi = W L^{-*} is computed to FP64 accuracy from the FP32 W and the
  *    FP64 L^{-*} on the FP16 tensor cores (error-free 8-bit integer slices of
  *    both operands, exact integer products, exact accumulation) and rounded

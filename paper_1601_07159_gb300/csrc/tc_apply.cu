@@ -8,7 +8,7 @@
 // 2018, with both parts scaled). hi and lo carry 22 to 23 bits of every value down to
 // 2^-18 of the row's largest (lo is then a normal FP16 number) and below that an absolute
 // error of 2^-40 of the largest. So what shares a scale matters: the gram product's
-// rows and columns are vectors; the outer product's rows are points (the largest value
+// rows and columns are vectors, scaled anew every 512 points; the outer product's rows are points (the largest value
 // of any orbital there), so that V_ACE psi keeps its relative accuracy where every
 // orbital is small, as in vacuum, and its columns are the bands' coefficients.
 // Three products hi hi + hi lo + lo hi are kept; the dropped lo lo is below
@@ -36,13 +36,13 @@
 // are added in FP32 registers while the next group's MMAs run. Every mbarrier wait
 // is bounded, as in tc_gemm.cu.
 //
-// Measured, TF32 split -> this: 48^3, 128 orbitals, 192 bands: gram 169 -> 94 us, outer
-// 188 -> 122 us, the new pass over the vectors for their largest values 48 us (5.9
-// TB/s), whole call 378 -> 294 us; 96^3, 1024 x 1536: 116 -> 79 ms (gram 38,
-// outer 39). With the MMAs and the conversion switched off the 48^3 loops still take 67
-// and 95 us (387 and 553 MB through L2, 5.8 TB/s): tile traffic bounds them, then the
-// chain convert - fence - barrier - issue of a chunk. Relative error against FP64 at
-// 48^3: 2.7e-6 -> 9.7e-7.
+// Measured, TF32 split -> this: 48^3, 128 orbitals, 192 bands: gram 169 -> 96 us, outer
+// 188 -> 100 us, the sweep over the vectors for their maxima 43 us (6.5 TB/s), whole
+// call 378 -> 278 us; 96^3, 1024 x 1536: 116 -> 71.4 ms (gram 37.5, outer 31.3, maxima 2.4).
+// With the MMAs and the conversion switched off the 48^3 loops take 67 us (gram) and 95
+// (outer, with a scale per value) (387 and 553 MB through L2, 5.8 TB/s): tile traffic
+// bounds them, then the chain convert - fence - barrier - issue of a chunk. Relative error
+// against FP64 at 48^3: 2.7e-6 -> 9.6e-7.
 #include <cstdint>
 #include <type_traits>
 #include <cuda.h>
@@ -85,7 +85,7 @@ template <int TN> struct Tile {
   static constexpr int G_STAGES = TN == 64 ? 4 : TN == 256 ? 2 : 3;
   static constexpr int G_RING = TN == 64 ? 6 : TN == 128 ? 5 : TN == 192 ? 3 : 4;   // what 227 KB hold
   static constexpr int G_SMEM = G_STAGES * G_STAGE + G_RING * G_RAW + 1024 + 128;
-  // outer: stages of A_hi, A_lo, a ring of four right operands, a raw ring of A
+  // outer: stages of A_hi, A_lo, a ring of right operands, a raw ring of A
   static constexpr int O_STAGE = 2 * A_TILE;
   static constexpr int O_B = 2 * B_TILE;
   static constexpr int O_RAW = TM * KC * 4;
@@ -106,6 +106,16 @@ __device__ __forceinline__ int scale_exp(unsigned m) {
   return e < 15 ? 126 : 141 - e;          // tiny vectors: 2^126 keeps them far from overflow
 }
 __device__ __forceinline__ float exp2i(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }   // |e| <= 126
+
+// Further powers of two for a vector's values within one 512-point segment, from the
+// biased exponents of the vector's and the segment's largest: in steps of 4, so that
+// vectors without large variation stay in one unit, and at most 36, so that sums over
+// all points in the units of two boosts stay below 2^123.
+__device__ __forceinline__ int exp_scale(int e) { return e == 255 ? 0 : e < 15 ? 126 : 141 - e; }
+__device__ __forceinline__ int boost(int ev, int es) {
+  if (ev == 0 || ev == 255) return 0;
+  return min((exp_scale(es) - exp_scale(ev)) & ~3, 36);
+}
 
 // one box of a 2D tensor map (x in floats, a multiple of 4; y a vector) to shared
 // memory; coordinates past the tensor read zero and count as bytes on `bar`
@@ -194,13 +204,15 @@ template <int TN> struct Stream {
 #pragma unroll
     for (int i = 0; i < Tile<TN>::NH; ++i) re[i] = im[i] = 0.f;
   }
-  // bounded wait for the MMAs of stage s, then the sums of a finished group
-  __device__ __forceinline__ bool settle(int s) {
+  // bounded wait for the MMAs of stage s, then the sums of a finished group, whose units
+  // `units` gives the sums so far
+  template <typename F> __device__ __forceinline__ bool settle(int s, F&& units) {
     if (!tc::mbar_wait(&bar[s], (phase >> s) & 1u, kWaitLimit)) return false;
     phase ^= 1u << s;
     issued &= ~(1u << s);
     const unsigned d = (drain >> (2 * s)) & 3u;
     if (d) {
+      units();
       tc::fence_after_sync();
       const uint32_t t = tmem + lane_col + (uint32_t)(TN * (d - 1));
       tmem_add<Tile<TN>::NH>(t, re);
@@ -234,28 +246,34 @@ template <int TN> __device__ __forceinline__ void teardown(uint32_t tmem) {
 
 // Largest |component| (as float bits, which order like the values; NaN is skipped) of
 // each vector, mx[0 .. na) for A and mx[na ..) for B, and of each point over the vectors
-// of A, pt[g]. Grid: (ya parts of `per` vectors of A and then those of B, 512-point
+// of A, pt[g]; the biased exponent of each vector's largest in each segment, sx[segment *
+// row + vector], with the vectors of B from `at_b` on. Grid: (ya parts of `per` vectors of A and then those of B, 512-point
 // segments). A warp takes a segment of one vector at a time, eight 16-byte loads in flight a
 // thread, and keeps the maxima of its points in registers; one sweep of the vectors,
 // bound by memory.
-constexpr int SEG = 512;
+constexpr int SEG = 512, kMaxPart = 64;
 __global__ void __launch_bounds__(256)
 maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B, int nb, long long ld, long long ng,
-              int per, int ya, unsigned* __restrict__ mx, unsigned* __restrict__ pt) {
+              int per, int ya, unsigned* __restrict__ mx, unsigned* __restrict__ pt, unsigned char* __restrict__ sx, int row, int at_b) {
+  __shared__ unsigned vm[kMaxPart];
   const bool first = (int)blockIdx.x < ya;               // a part of A
   const int count = first ? na : nb, v0 = ((int)blockIdx.x - (first ? 0 : ya)) * per;
   const int v1 = v0 + per < count ? v0 + per : count;
   const float2* X = first ? A : B;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long n = ng / 2, i0 = (long long)blockIdx.y * (SEG / 2);   // float4 units: N_g is even on every grid
+  int off[8];                                            // past the grid's end: its last points again
   float2 p[8];
 #pragma unroll
-  for (int u = 0; u < 8; ++u) p[u] = make_float2(0.f, 0.f);
+  for (int u = 0; u < 8; ++u) {
+    off[u] = i0 + lane + 32 * u < n ? lane + 32 * u : (int)(n - 1 - i0);
+    p[u] = make_float2(0.f, 0.f);
+  }
   for (int v = v0 + w; v < v1; v += 8) {
-    const float4* x = reinterpret_cast<const float4*>(X + (long long)v * ld) + i0 + lane;
+    const float4* x = reinterpret_cast<const float4*>(X + (long long)v * ld) + i0;
     float4 t[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = i0 + lane + 32 * u < n ? x[32 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int u = 0; u < 8; ++u) t[u] = x[off[u]];
     float m = 0.f;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
@@ -264,13 +282,21 @@ maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B
       m = fmaxf(m, fmaxf(a, b));
     }
     const unsigned r = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-    if (lane == 0) atomicMax(mx + (first ? v : na + v), r);
+    if (lane == 0) vm[v - v0] = r;
+  }
+  __shared__ float2 red[8][SEG / 2];
+  if (first) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) red[w][lane + 32 * u] = p[u];
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < v1 - v0) {
+    const unsigned r = vm[threadIdx.x];
+    const int v = v0 + threadIdx.x;
+    atomicMax(mx + (first ? v : na + v), r);
+    sx[(long long)blockIdx.y * row + (first ? v : at_b + v)] = (unsigned char)(r >> 23);
   }
   if (!first) return;
-  __shared__ float2 red[8][SEG / 2];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) red[w][lane + 32 * u] = p[u];
-  __syncthreads();
   const int i = threadIdx.x;
   float2 q = red[0][i];
 #pragma unroll
@@ -288,10 +314,17 @@ maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B
 // 128-byte swizzle: 16-byte granule g of row r lies at g ^ (r & 7)) arrive by two TMA
 // loads. Thread t owns row 8 (t / 32) + t % 8 and granules q and q + 4, q = (t / 8) % 4:
 // its loads are conflict-free and its stores fill 128 contiguous bytes per 16 lanes.
+// Scales are those of the vectors times each segment's boost, so that overlaps far below
+// the vectors' largest values keep their accuracy: accumulator groups end where
+// segments do, and when a segment's boosts differ from those of the sums so far, the
+// sums are taken to its units first (a multiplication by a power of two). The split's
+// sums are left in the units of the vectors. A segment's
+// exponents arrive with its first chunk.
 template <int TN>
 __global__ void __launch_bounds__(Tile<TN>::G_THREADS, 1)
 gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_constant__ CUtensorMap B, int nb, long long ng,
-              const unsigned* __restrict__ mx, float2* __restrict__ part, long long chunk, int* status) {
+              const unsigned* __restrict__ mx, const unsigned char* __restrict__ sx, int row, int at_b,
+              float2* __restrict__ part, long long chunk, int* status) {
   using T = Tile<TN>;
   constexpr int BB = T::BB, NH = T::NH, R = T::G_RING, ST = T::G_STAGES;
   extern __shared__ unsigned char smem_raw[];
@@ -299,7 +332,11 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
   unsigned char* ring = base + ST * T::G_STAGE;
   uint64_t* bar = reinterpret_cast<uint64_t*>(ring + R * T::G_RAW);   // [0, ST): MMAs of a stage; then R: a chunk landed; then ST: a stage stored
   __shared__ volatile int s_fail;
+  // biased exponents of the tile's 128 rows and BB columns: of the vectors' largest
+  // values, and of their largest in the even and the odd segments
+  __shared__ __align__(16) unsigned char s_ev[TM + BB], s_es[2][TM + BB];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int a0 = blockIdx.x * TM, b0 = blockIdx.y * BB;
   if (tid == 0) s_fail = 0;
   Stream<TN> S;
   S.bar = bar;
@@ -307,22 +344,32 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
   S.tmem = setup<TN>(bar, ST + R, reinterpret_cast<uint32_t*>(bar + 2 * ST + R), IW ? ST : 0);
   S.lane_col = ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(NH * (w >> 2));
 
-  const int a0 = blockIdx.x * TM, b0 = blockIdx.y * BB;
   const long long g_begin = (long long)blockIdx.z * chunk;
   const long long g_end = g_begin + chunk < ng ? g_begin + chunk : ng;
   const int nchunks = g_end > g_begin ? (int)((g_end - g_begin + KC / 2 - 1) / (KC / 2)) : 0;
   const int r = (w << 3) | (tid & 7), q = (tid >> 3) & 3;
   const bool arow = a0 + r < na, brow = r < BB && b0 + r < nb;
   const bool bthr = r < BB;                              // uniform in a warp
-  const float sa = arow ? exp2i(scale_exp(mx[a0 + r])) : 0.f, sb = brow ? exp2i(scale_exp(mx[na + b0 + r])) : 0.f;
+  constexpr int SC = 2 * SEG / KC, SG = SC / kGroup;     // chunks and groups per segment
+  const unsigned c0 = (unsigned)(g_begin / (KC / 2));    // segments and groups count from the grid's first point
+  auto group_start = [&](int c) { return c == 0 || (c0 + c) % kGroup == 0; };
+  auto buffer = [&](int c) { return (int)((c0 + c) / kGroup & 1); };
+  auto boost_of = [&](int i, int segment) { return boost(s_ev[i], s_es[segment & 1][i]); };
   auto fetch = [&](int c) {
     if (c < nchunks) {
       const int slot = c % R, x = (int)(2 * g_begin) + KC * c;
       uint64_t* fb = bar + ST + slot;
       unsigned char* d = ring + slot * T::G_RAW;
-      tc::mbar_arrive_expect_tx(fb, (unsigned)T::G_RAW);
+      const bool start = c == 0 || (c0 + c) % SC == 0;   // a segment: its exponents come with its first chunk
+      tc::mbar_arrive_expect_tx(fb, (unsigned)(T::G_RAW + (start ? TM + BB : 0)));
       load_box(d, A, x, a0, fb);
       load_box(d + TM * KC * 4, B, x, b0, fb);
+      if (start) {
+        const int e = (int)((c0 + c) / SC);
+        const unsigned char* src = sx + (long long)e * row;
+        tc::bulk_g2s(s_es[e & 1], src + a0, TM, fb);
+        tc::bulk_g2s(s_es[e & 1] + TM, src + at_b + b0, BB, fb);
+      }
     }
   };
   if (IW && w >= THREADS / 32) {                         // ---- the issuing warp (and three idle ones)
@@ -337,7 +384,7 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
         if (!tc::mbar_wait(bar + ST + R + s, (unsigned)(c / ST) & 1u, kWaitLimit)) break;
         tc::fence_after_sync();
         const uint32_t sa0 = smem_u32(base + s * T::G_STAGE);
-        issue_chunk<TN>(S.tmem + (uint32_t)(TN * ((c / kGroup) & 1)), sa0, sa0 + 2 * A_TILE, c % kGroup == 0);
+        issue_chunk<TN>(S.tmem + (uint32_t)(TN * buffer(c)), sa0, sa0 + 2 * A_TILE, group_start(c));
         tc::mma_commit(&bar[s]);
         fetch(c + R);
       }
@@ -351,7 +398,36 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
   if (TN == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");   // 512 x 112 + 128 x 24 of 640 x 96 registers
   if (!IW && tid == 32)
     for (int c = 0; c < R - 1; ++c) fetch(c);
+  if (tid < TM + BB) {
+    const int v = tid < TM ? a0 + tid : na + b0 + tid - TM;
+    s_ev[tid] = v < (tid < TM ? na : na + nb) ? (unsigned char)(mx[v] >> 23) : 0;
+  }
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
   S.zero();
+  // the sums so far into the units of `to` (< 0: of the vectors) from those of segment `from`
+  const int lrow = 32 * (w & 3) + lane, lcol = NH * (w >> 2) + lane;   // this lane's row, and (lanes below NH) a column
+  auto rescale = [&](int from, int to) {
+    int db = -boost_of(lrow, from), dc = lane < NH ? -boost_of(TM + lcol, from) : 0;
+    if (to >= 0) {
+      db += boost_of(lrow, to);
+      if (lane < NH) dc += boost_of(TM + lcol, to);
+    }
+    if (__any_sync(0xffffffffu, (db | dc) != 0)) {
+#pragma unroll
+      for (int j = 0; j < NH; ++j) {
+        const float f = exp2i(db + __shfl_sync(0xffffffffu, dc, j));
+        S.re[j] *= f;
+        S.im[j] *= f;
+      }
+    }
+  };
+  unsigned group = c0 / kGroup;                          // the next group to add
+  auto units = [&]() {
+    if (group % SG == 0 && group > c0 / kGroup) rescale((int)(group / SG) - 1, (int)(group / SG));
+    ++group;
+  };
+  int fresh = 0;                                         // chunks left in this segment
+  float sa = 0.f, sb = 0.f;
   const int o = tile_off(r, 4 * q);
   constexpr int IM = (BB >> 3) * SBO;                    // rows BB ..: (im, -re)
   const int g0 = r * 128 + ((q ^ (r & 7)) << 4), g1 = g0 ^ 64;   // the granules in a raw tile
@@ -362,6 +438,12 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
     if (!IW && tid == 32) fetch(c + R - 1);               // into the slot that chunk c - 1 left
     if (!tc::mbar_wait(bar + ST + slot, (lphase >> slot) & 1u, kWaitLimit)) s_fail = 1;
     else lphase ^= 1u << slot;
+    if (fresh-- == 0) {
+      const int e = (int)((c0 + c) / SC);
+      fresh = SC - 1 - (int)((c0 + c) % SC);
+      if (arow) sa = exp2i(exp_scale(s_ev[r]) + boost_of(r, e));
+      if (brow) sb = exp2i(exp_scale(s_ev[TM + r]) + boost_of(TM + r, e));
+    }
     const unsigned char* raw = ring + slot * T::G_RAW;
     unsigned char* st = base + s * T::G_STAGE + o;
     uint2 ah[2], al[2], bh[2], bl[2];
@@ -371,7 +453,7 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
       split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g0), sb, bh[0], bl[0]);
       split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g1), sb, bh[1], bl[1]);
     }
-    if (((S.issued >> s) & 1u) && !S.settle(s)) s_fail = 1;   // the MMAs of chunk c - ST read this stage
+    if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;   // the MMAs of chunk c - ST read this stage
 #pragma unroll
     for (int i = 0; i < 2; ++i) {                        // granule i: K values 4 q + 16 i ..
       *reinterpret_cast<uint2*>(st + i * 256) = ah[i];
@@ -388,7 +470,7 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
       }
     }
     tc::fence_async_smem();
-    const int buf = (c / kGroup) & 1;
+    const int buf = buffer(c);
     if constexpr (IW) {
       __syncwarp();
       if (lane == 0)
@@ -406,20 +488,21 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
       if (tid == 0) {
         const uint32_t sa0 = smem_u32(base + s * T::G_STAGE);
         tc::fence_after_sync();
-        issue_chunk<TN>(S.tmem + (uint32_t)(TN * buf), sa0, sa0 + 2 * A_TILE, c % kGroup == 0);
+        issue_chunk<TN>(S.tmem + (uint32_t)(TN * buf), sa0, sa0 + 2 * A_TILE, group_start(c));
         tc::mma_commit(&bar[s]);
       }
     }
     S.issued |= 1u << s;
-    if (c % kGroup == kGroup - 1 || c == nchunks - 1) S.drain |= (1u + (unsigned)buf) << (2 * s);
+    if ((c0 + c) % kGroup == kGroup - 1 || c == nchunks - 1) S.drain |= (1u + (unsigned)buf) << (2 * s);
   }
   for (int i = 0; i < ST; ++i) {                         // the last commits, in chunk order
     const int s = (nchunks + i) % ST;
-    if (((S.issued >> s) & 1u) && !S.settle(s)) s_fail = 1;
+    if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;
   }
   if (!IW && !ok)                                        // copies in flight (bounded)
     for (int i = 0; i < R; ++i) tc::mbar_wait(bar + ST + i, (lphase >> i) & 1u, 1u << 16);
-  const int a = a0 + 32 * (w & 3) + lane, bq = b0 + NH * (w >> 2);
+  if (nchunks > 0) rescale((int)((c0 + nchunks - 1) / SC), -1);
+  const int a = a0 + lrow, bq = b0 + NH * (w >> 2);
   if (ok && a < na) {
     float2* out = part + ((long long)blockIdx.z * na + a) * nb + bq;
 #pragma unroll
@@ -618,7 +701,7 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nb, long long ld, long
   int due0 = -1, due1 = -1;                              // tile that ends with the pending commit of stage 0, 1
   unsigned lphase = 0;                                   // parities of the landing barriers
   auto finish = [&](int s) {                             // the pending commit of stage s, and the stores that it ends
-    if (!S.settle(s)) {
+    if (!S.settle(s, [] {})) {
       s_fail = 1;
       return;
     }
@@ -688,7 +771,7 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nb, long long ld, long
     }
   } else {
     for (int s = 0; s < 2; ++s)
-      if ((S.issued >> s) & 1u) S.settle(s);
+      if ((S.issued >> s) & 1u) S.settle(s, [] {});
     for (int i = 0; i < R; ++i)                          // copies in flight (bounded)
       tc::mbar_wait(bar + 2 + i, (lphase >> i) & 1u, 1u << 16);
   }
@@ -752,13 +835,15 @@ int splits_for(long long ng, int na, int nb, long long cap) {
   return (int)best;
 }
 
-// Scratch layout: vector and point maxima, column exponents, C, and the split sums, which
-// the right operand overwrites once they are reduced. The splits are those that fit `budget`
+// Scratch layout: vector, point and segment maxima, column exponents, C, and the split
+// sums, which the right operand overwrites once they are reduced. The splits are those that fit `budget`
 // bytes: the plan's workspace holds what the TF32 products take, or `least` (one split)
-// if that is more, and the maxima of the points (`tables`) beside it.
+// if that is more, and the maxima of the points and segments (`tables`) beside it.
 struct Scratch {
-  unsigned* mx;      // vector maxima, then (at pt) point maxima
-  unsigned* pt;
+  unsigned* mx;      // vector maxima
+  unsigned* pt;      // point maxima
+  unsigned char* sx; // segment exponents: rows of `row` bytes, Psi's from at_b on
+  int row, at_b;
   int* colexp;
   unsigned char* Bs;
   float2* C;
@@ -774,7 +859,11 @@ Scratch scratch(char* base, long long ng, int n, int nb, size_t budget) {
   const size_t nbt = (size_t)(nb + bb - 1) / bb, nch = (size_t)(n + 15) / 16;
   s.mx = (unsigned*)take((size_t)(n + nb) * sizeof(unsigned));
   s.pt = (unsigned*)take((size_t)ng * sizeof(unsigned));   // behind mx: one memset clears both
-  s.tables = align256((size_t)ng * sizeof(unsigned));
+  s.at_b = (n + TM - 1) / TM * TM;                       // rows of whole tiles: a tile's bytes come by bulk copies
+  s.row = s.at_b + (int)(nbt * bb);
+  const size_t bytes = (size_t)((ng + SEG - 1) / SEG) * s.row;
+  s.sx = (unsigned char*)take(bytes);
+  s.tables = align256((size_t)ng * sizeof(unsigned)) + align256(bytes);
   s.colexp = (int*)take((size_t)nb * sizeof(int));
   s.C = (float2*)take((size_t)n * nb * sizeof(float2));
   s.part = (float2*)take(0);
@@ -820,11 +909,12 @@ bool apply_tc_prepare() {
   return cudaGetLastError() == cudaSuccess;
 }
 
-// Six launches against four: on grids below 2^16 points and 7 2^18 values in all vectors
-// the TF32 products of tc_gemm.cu are the faster on some shapes (graph replay, TF32 ->
-// this: 24^3, 30 + 30 vectors 25.4 -> 28.3 us; 60 + 60 32.2 -> 33.4; above the line 36^3, 16 +
-// 24: 46.0 -> 39.6; 12^3, 500 + 700: 271 -> 143; 24^3, 100 + 100: 54.6 -> 49.6; 48^3, 4 + 2:
-// 78.3 -> 61.9; 16 + 24: 85.5 -> 65.0; 96^3, 1 + 1: 523 -> 347).
+// Six launches against four: the TF32 products of tc_gemm.cu are the faster on the
+// smallest calls (graph replay, TF32 -> this: 24^3, 10 + 10 vectors 22.6 -> 23.3 us; 30 + 30
+// 24.8 -> 24.0; 60 + 60 32.3 -> 30.7; 36^3, 4 + 4 42.7 -> 35.7). Above the line: 36^3, 16 +
+// 24: 46.1 -> 36.6; 12^3, 500 + 700: 271 -> 136; 24^3, 100 + 100: 55.2 -> 48.2; 48^3, 4 + 2:
+// 77.6 -> 58.5; 16 + 24: 85.6 -> 61.2; 1024 + 1: 922 -> 645; 96^3, 1 + 1: 524 -> 341. The line was
+// drawn before the sweep for the maxima took 43 us in place of 48, and could lie lower.
 bool apply_tc_faster(long long ng, int n, int nb) {
   return ng >= (1LL << 16) || ng * ((long long)n + nb) >= (7LL << 18);
 }
@@ -848,9 +938,9 @@ int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld
   // eight to 64 vectors per block (one to eight per warp), by what gives eight blocks per SM
   const long long segs = (ng + SEG - 1) / SEG;
   long long per = (segs * ((long long)n + nb) / (8 * 152) + 7) / 8 * 8;
-  per = per < 8 ? 8 : per > 64 ? 64 : per;
+  per = per < 8 ? 8 : per > kMaxPart ? kMaxPart : per;
   const int ya = (int)((n + per - 1) / per), yb = (int)((nb + per - 1) / per);
-  maxima_kernel<<<dim3(ya + yb, (unsigned)segs), 256, 0, st>>>(x, n, psi, nb, ld, ng, (int)per, ya, s.mx, s.pt);
+  maxima_kernel<<<dim3(ya + yb, (unsigned)segs), 256, 0, st>>>(x, n, psi, nb, ld, ng, (int)per, ya, s.mx, s.pt, s.sx, s.row, s.at_b);
   const int splits = s.splits, nch = (n + 15) / 16;
   long long chunk = (ng + splits - 1) / splits;
   chunk = (chunk + KC / 2 - 1) / (KC / 2) * (KC / 2);
@@ -858,8 +948,8 @@ int launch_apply_tc(const void* Xi, int n, const void* Psi, int nb, long long ld
     constexpr int TN = decltype(t)::value;
     using T = Tile<TN>;
     const int nbt = (nb + T::BB - 1) / T::BB;
-    gram16_kernel<TN><<<dim3((n + TM - 1) / TM, nbt, splits), T::G_THREADS, T::G_SMEM, st>>>(xg, n, qg, nb, ng, s.mx, s.part,
-                                                                                     chunk, status);
+    gram16_kernel<TN><<<dim3((n + TM - 1) / TM, nbt, splits), T::G_THREADS, T::G_SMEM, st>>>(xg, n, qg, nb, ng, s.mx, s.sx,
+                                                                                     s.row, s.at_b, s.part, chunk, status);
     const long long total = (long long)n * nb;
     int ways = 8;
     while (ways > 1 && (ways > splits || total * ways > 152LL * 2048)) ways /= 2;

@@ -81,3 +81,43 @@ def test_accuracy_where_every_orbital_is_small(ace, prec, nocc, nb):
     rng = np.random.default_rng(nocc)
     xi, psi = _near(rng, nocc, 10.0), _near(rng, nb, 10.0)
     assert _point_error(_apply(_plan(ace, nocc, prec=prec), xi, psi), xi, psi) < TOL
+
+
+@pytest.mark.parametrize("decades", [5.0, 10.0])
+@pytest.mark.parametrize("nocc,nb", [(5, 3), (17, 40), (140, 100)])
+@pytest.mark.parametrize("prec", ["default", "split_tf32"])
+def test_accuracy_of_overlaps_in_the_tails(ace, prec, nocc, nb, decades):
+    """Bands that grow where the orbitals decay: every point contributes alike to C, from
+    values far below the largest of both vectors."""
+    rng = np.random.default_rng(nocc + 1)
+    xi, psi = _near(rng, nocc, decades), _near(rng, nb, decades, axis_up=True)
+    got, want = _apply(_plan(ace, nocc, prec=prec), xi, psi), _want(xi, psi)
+    err = np.linalg.norm((got - want).reshape(nb, -1), axis=1) / np.linalg.norm(want.reshape(nb, -1), axis=1)
+    print(prec, nocc, nb, decades, err.max())
+    assert err.max() < TOL
+
+
+def test_vectors_of_subnormal_size(ace):
+    """Orbitals below FP32's normal range on bands near its top: every intermediate
+    leaves the range, the result does not (and carries the subnormals' spacing, 2^-149)."""
+    rng = np.random.default_rng(5)
+    xi, psi = _random(rng, 6) * np.float32(1e-39), _random(rng, 5) * np.float32(5e37)
+    got, want = _apply(_plan(ace, 6), xi, psi), _want(xi, psi)
+    err = np.linalg.norm((got - want).reshape(5, -1), axis=1)
+    assert (err < TOL * np.linalg.norm(want.reshape(5, -1), axis=1) + 2.0 ** -149 * np.sqrt(2 * got[0].size)).all()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_nonfinite_values_stay_in_their_band(ace, bad):
+    """A band with a NaN or an infinity has no finite result; the others are those
+    without it. In an orbital it reaches every band."""
+    rng = np.random.default_rng(6)
+    xi, psi = _random(rng, 20), _random(rng, 30)
+    clean = _apply(_plan(ace, 20), xi, psi)
+    psi[7, 3, 5, 9] = bad
+    got = _apply(_plan(ace, 20), xi, psi)
+    assert not np.isfinite(got[7]).any()
+    assert np.array_equal(np.delete(got, 7, 0), np.delete(clean, 7, 0))
+    psi[7, 3, 5, 9] = 0
+    xi[4, 1, 2, 3] = bad
+    assert not np.isfinite(_apply(_plan(ace, 20), xi, psi)).any()
