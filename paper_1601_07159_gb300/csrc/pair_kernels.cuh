@@ -265,7 +265,7 @@ template <int NX, int NY> constexpr int kMaxLine = NX > NY ? NX : NY;
 // 5.0, 36^3 7.3 -> 6.6 ps per pair point; FP64 24^3 242 -> 170). At most 96 KB.
 template <typename R, int NX, int NY> __host__ __device__ constexpr int plane_items() {
   constexpr int ML = kMaxLine<NX, NY>;
-    constexpr int by_threads = (128 / ML) > 0 ? (128 / ML) : 1;
+  constexpr int by_threads = (128 / ML) > 0 ? (128 / ML) : 1;
   constexpr int by_smem = (96 * 1024) / (NY * (NX + 1) * (int)sizeof(cplx<R>));
   constexpr int v = by_threads < by_smem ? by_threads : by_smem;
   return v > 0 ? v : 1;

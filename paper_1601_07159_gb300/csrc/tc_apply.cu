@@ -254,7 +254,8 @@ template <int TN> __device__ __forceinline__ void teardown(uint32_t tmem) {
 constexpr int SEG = 512, kMaxPart = 64;
 __global__ void __launch_bounds__(256)
 maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B, int nb, long long ld, long long ng,
-              int per, int ya, unsigned* __restrict__ mx, unsigned* __restrict__ pt, unsigned char* __restrict__ sx, int row, int at_b) {
+              int per, int ya, unsigned* __restrict__ mx, unsigned* __restrict__ pt, unsigned char* __restrict__ sx,
+              int row, int at_b) {
   __shared__ unsigned vm[kMaxPart];
   const bool first = (int)blockIdx.x < ya;               // a part of A
   const int count = first ? na : nb, v0 = ((int)blockIdx.x - (first ? 0 : ya)) * per;
@@ -330,7 +331,8 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* ring = base + ST * T::G_STAGE;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(ring + R * T::G_RAW);   // [0, ST): MMAs of a stage; then R: a chunk landed; then ST: a stage stored
+  // barriers: ST for the MMAs of a stage, R for a landed chunk, ST for a stored stage
+  uint64_t* bar = reinterpret_cast<uint64_t*>(ring + R * T::G_RAW);
   __shared__ volatile int s_fail;
   // biased exponents of the tile's 128 rows and BB columns: of the vectors' largest
   // values, and of their largest in the even and the odd segments
@@ -395,122 +397,122 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
       }
     }
   } else {                                               // ---- the working warps
-  if (TN == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");   // 512 x 112 + 128 x 24 of 640 x 96 registers
-  if (!IW && tid == 32)
-    for (int c = 0; c < R - 1; ++c) fetch(c);
-  if (tid < TM + BB) {
-    const int v = tid < TM ? a0 + tid : na + b0 + tid - TM;
-    s_ev[tid] = v < (tid < TM ? na : na + nb) ? (unsigned char)(mx[v] >> 23) : 0;
-  }
-  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
-  S.zero();
-  // the sums so far into the units of `to` (< 0: of the vectors) from those of segment `from`
-  const int lrow = 32 * (w & 3) + lane, lcol = NH * (w >> 2) + lane;   // this lane's row, and (lanes below NH) a column
-  auto rescale = [&](int from, int to) {
-    int db = -boost_of(lrow, from), dc = lane < NH ? -boost_of(TM + lcol, from) : 0;
-    if (to >= 0) {
-      db += boost_of(lrow, to);
-      if (lane < NH) dc += boost_of(TM + lcol, to);
+    if (TN == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");   // 512 x 112 + 128 x 24 of 640 x 96 registers
+    if (!IW && tid == 32)
+      for (int c = 0; c < R - 1; ++c) fetch(c);
+    if (tid < TM + BB) {
+      const int v = tid < TM ? a0 + tid : na + b0 + tid - TM;
+      s_ev[tid] = v < (tid < TM ? na : na + nb) ? (unsigned char)(mx[v] >> 23) : 0;
     }
-    if (__any_sync(0xffffffffu, (db | dc) != 0)) {
+    asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+    S.zero();
+    // the sums so far into the units of `to` (< 0: of the vectors) from those of segment `from`
+    const int lrow = 32 * (w & 3) + lane, lcol = NH * (w >> 2) + lane;   // this lane's row, and (lanes below NH) a column
+    auto rescale = [&](int from, int to) {
+      int db = -boost_of(lrow, from), dc = lane < NH ? -boost_of(TM + lcol, from) : 0;
+      if (to >= 0) {
+        db += boost_of(lrow, to);
+        if (lane < NH) dc += boost_of(TM + lcol, to);
+      }
+      if (__any_sync(0xffffffffu, (db | dc) != 0)) {
 #pragma unroll
-      for (int j = 0; j < NH; ++j) {
-        const float f = exp2i(db + __shfl_sync(0xffffffffu, dc, j));
-        S.re[j] *= f;
-        S.im[j] *= f;
+        for (int j = 0; j < NH; ++j) {
+          const float f = exp2i(db + __shfl_sync(0xffffffffu, dc, j));
+          S.re[j] *= f;
+          S.im[j] *= f;
+        }
       }
-    }
-  };
-  unsigned group = c0 / kGroup;                          // the next group to add
-  auto units = [&]() {
-    if (group % SG == 0 && group > c0 / kGroup) rescale((int)(group / SG) - 1, (int)(group / SG));
-    ++group;
-  };
-  int fresh = 0;                                         // chunks left in this segment
-  float sa = 0.f, sb = 0.f;
-  const int o = tile_off(r, 4 * q);
-  constexpr int IM = (BB >> 3) * SBO;                    // rows BB ..: (im, -re)
-  const int g0 = r * 128 + ((q ^ (r & 7)) << 4), g1 = g0 ^ 64;   // the granules in a raw tile
-  bool ok = true;
-  unsigned lphase = 0;                                   // parities of the landing barriers
-  for (int c = 0; c < nchunks; ++c) {
-    const int s = c % ST, slot = c % R;
-    if (!IW && tid == 32) fetch(c + R - 1);               // into the slot that chunk c - 1 left
-    if (!tc::mbar_wait(bar + ST + slot, (lphase >> slot) & 1u, kWaitLimit)) s_fail = 1;
-    else lphase ^= 1u << slot;
-    if (fresh-- == 0) {
-      const int e = (int)((c0 + c) / SC);
-      fresh = SC - 1 - (int)((c0 + c) % SC);
-      if (arow) sa = exp2i(exp_scale(s_ev[r]) + boost_of(r, e));
-      if (brow) sb = exp2i(exp_scale(s_ev[TM + r]) + boost_of(TM + r, e));
-    }
-    const unsigned char* raw = ring + slot * T::G_RAW;
-    unsigned char* st = base + s * T::G_STAGE + o;
-    uint2 ah[2], al[2], bh[2], bl[2];
-    split4(*reinterpret_cast<const float4*>(raw + g0), sa, ah[0], al[0]);
-    split4(*reinterpret_cast<const float4*>(raw + g1), sa, ah[1], al[1]);
-    if (bthr) {
-      split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g0), sb, bh[0], bl[0]);
-      split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g1), sb, bh[1], bl[1]);
-    }
-    if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;   // the MMAs of chunk c - ST read this stage
+    };
+    unsigned group = c0 / kGroup;                          // the next group to add
+    auto units = [&]() {
+      if (group % SG == 0 && group > c0 / kGroup) rescale((int)(group / SG) - 1, (int)(group / SG));
+      ++group;
+    };
+    int fresh = 0;                                         // chunks left in this segment
+    float sa = 0.f, sb = 0.f;
+    const int o = tile_off(r, 4 * q);
+    constexpr int IM = (BB >> 3) * SBO;                    // rows BB ..: (im, -re)
+    const int g0 = r * 128 + ((q ^ (r & 7)) << 4), g1 = g0 ^ 64;   // the granules in a raw tile
+    bool ok = true;
+    unsigned lphase = 0;                                   // parities of the landing barriers
+    for (int c = 0; c < nchunks; ++c) {
+      const int s = c % ST, slot = c % R;
+      if (!IW && tid == 32) fetch(c + R - 1);               // into the slot that chunk c - 1 left
+      if (!tc::mbar_wait(bar + ST + slot, (lphase >> slot) & 1u, kWaitLimit)) s_fail = 1;
+      else lphase ^= 1u << slot;
+      if (fresh-- == 0) {
+        const int e = (int)((c0 + c) / SC);
+        fresh = SC - 1 - (int)((c0 + c) % SC);
+        if (arow) sa = exp2i(exp_scale(s_ev[r]) + boost_of(r, e));
+        if (brow) sb = exp2i(exp_scale(s_ev[TM + r]) + boost_of(TM + r, e));
+      }
+      const unsigned char* raw = ring + slot * T::G_RAW;
+      unsigned char* st = base + s * T::G_STAGE + o;
+      uint2 ah[2], al[2], bh[2], bl[2];
+      split4(*reinterpret_cast<const float4*>(raw + g0), sa, ah[0], al[0]);
+      split4(*reinterpret_cast<const float4*>(raw + g1), sa, ah[1], al[1]);
+      if (bthr) {
+        split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g0), sb, bh[0], bl[0]);
+        split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g1), sb, bh[1], bl[1]);
+      }
+      if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;   // the MMAs of chunk c - ST read this stage
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {                        // granule i: K values 4 q + 16 i ..
-      *reinterpret_cast<uint2*>(st + i * 256) = ah[i];
-      *reinterpret_cast<uint2*>(st + A_TILE + i * 256) = al[i];
-    }
-    if (bthr) {
+      for (int i = 0; i < 2; ++i) {                        // granule i: K values 4 q + 16 i ..
+        *reinterpret_cast<uint2*>(st + i * 256) = ah[i];
+        *reinterpret_cast<uint2*>(st + A_TILE + i * 256) = al[i];
+      }
+      if (bthr) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        unsigned char* b = st + 2 * A_TILE + i * 256;
-        *reinterpret_cast<uint2*>(b) = bh[i];
-        *reinterpret_cast<uint2*>(b + T::B_TILE) = bl[i];
-        *reinterpret_cast<uint2*>(b + IM) = make_uint2(swap_neg(bh[i].x), swap_neg(bh[i].y));
-        *reinterpret_cast<uint2*>(b + T::B_TILE + IM) = make_uint2(swap_neg(bl[i].x), swap_neg(bl[i].y));
+        for (int i = 0; i < 2; ++i) {
+          unsigned char* b = st + 2 * A_TILE + i * 256;
+          *reinterpret_cast<uint2*>(b) = bh[i];
+          *reinterpret_cast<uint2*>(b + T::B_TILE) = bl[i];
+          *reinterpret_cast<uint2*>(b + IM) = make_uint2(swap_neg(bh[i].x), swap_neg(bh[i].y));
+          *reinterpret_cast<uint2*>(b + T::B_TILE + IM) = make_uint2(swap_neg(bl[i].x), swap_neg(bl[i].y));
+        }
       }
+      tc::fence_async_smem();
+      const int buf = buffer(c);
+      if constexpr (IW) {
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar + ST + R + s)) : "memory");
+        if (s_fail) {
+          ok = false;
+          break;
+        }
+      } else {
+        __syncthreads();
+        if (s_fail) {
+          ok = false;
+          break;
+        }
+        if (tid == 0) {
+          const uint32_t sa0 = smem_u32(base + s * T::G_STAGE);
+          tc::fence_after_sync();
+          issue_chunk<TN>(S.tmem + (uint32_t)(TN * buf), sa0, sa0 + 2 * A_TILE, group_start(c));
+          tc::mma_commit(&bar[s]);
+        }
+      }
+      S.issued |= 1u << s;
+      if ((c0 + c) % kGroup == kGroup - 1 || c == nchunks - 1) S.drain |= (1u + (unsigned)buf) << (2 * s);
     }
-    tc::fence_async_smem();
-    const int buf = buffer(c);
-    if constexpr (IW) {
-      __syncwarp();
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar + ST + R + s)) : "memory");
-      if (s_fail) {
-        ok = false;
-        break;
-      }
-    } else {
-      __syncthreads();
-      if (s_fail) {
-        ok = false;
-        break;
-      }
-      if (tid == 0) {
-        const uint32_t sa0 = smem_u32(base + s * T::G_STAGE);
-        tc::fence_after_sync();
-        issue_chunk<TN>(S.tmem + (uint32_t)(TN * buf), sa0, sa0 + 2 * A_TILE, group_start(c));
-        tc::mma_commit(&bar[s]);
-      }
+    for (int i = 0; i < ST; ++i) {                         // the last commits, in chunk order
+      const int s = (nchunks + i) % ST;
+      if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;
     }
-    S.issued |= 1u << s;
-    if ((c0 + c) % kGroup == kGroup - 1 || c == nchunks - 1) S.drain |= (1u + (unsigned)buf) << (2 * s);
-  }
-  for (int i = 0; i < ST; ++i) {                         // the last commits, in chunk order
-    const int s = (nchunks + i) % ST;
-    if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;
-  }
-  if (!IW && !ok)                                        // copies in flight (bounded)
-    for (int i = 0; i < R; ++i) tc::mbar_wait(bar + ST + i, (lphase >> i) & 1u, 1u << 16);
-  if (nchunks > 0) rescale((int)((c0 + nchunks - 1) / SC), -1);
-  const int a = a0 + lrow, bq = b0 + NH * (w >> 2);
-  if (ok && a < na) {
-    float2* out = part + ((long long)blockIdx.z * na + a) * nb + bq;
+    if (!IW && !ok)                                        // copies in flight (bounded)
+      for (int i = 0; i < R; ++i) tc::mbar_wait(bar + ST + i, (lphase >> i) & 1u, 1u << 16);
+    if (nchunks > 0) rescale((int)((c0 + nchunks - 1) / SC), -1);
+    const int a = a0 + lrow, bq = b0 + NH * (w >> 2);
+    if (ok && a < na) {
+      float2* out = part + ((long long)blockIdx.z * na + a) * nb + bq;
 #pragma unroll
-    for (int j = 0; j < NH; ++j)
-      if (bq + j < nb) out[j] = make_float2(S.re[j], S.im[j]);
+      for (int j = 0; j < NH; ++j)
+        if (bq + j < nb) out[j] = make_float2(S.re[j], S.im[j]);
+    }
+    if (!ok) s_fail = 1;
   }
-  if (!ok) s_fail = 1;
-  }   // working warps
   __syncthreads();
   if (s_fail && tid == 0) {
     status[0] = -6;   // ACE_ERR_TIMEOUT
@@ -913,7 +915,7 @@ bool apply_tc_prepare() {
 // smallest calls (graph replay, TF32 -> this: 24^3, 10 + 10 vectors 22.6 -> 23.3 us; 30 + 30
 // 24.8 -> 24.0; 60 + 60 32.3 -> 30.7; 36^3, 4 + 4 42.7 -> 35.7). Above the line: 36^3, 16 +
 // 24: 46.1 -> 36.6; 12^3, 500 + 700: 271 -> 136; 24^3, 100 + 100: 55.2 -> 48.2; 48^3, 4 + 2:
-// 77.6 -> 58.5; 16 + 24: 85.6 -> 61.2; 1024 + 1: 922 -> 645; 96^3, 1 + 1: 524 -> 341. The line was
+// 77.6 -> 58.5; 16 + 24: 85.6 -> 61.2; 1024 + 1: 922 -> 656; 96^3, 1 + 1: 524 -> 341. The line was
 // drawn before the sweep for the maxima took 43 us in place of 48, and could lie lower.
 bool apply_tc_faster(long long ng, int n, int nb) {
   return ng >= (1LL << 16) || ng * ((long long)n + nb) >= (7LL << 18);

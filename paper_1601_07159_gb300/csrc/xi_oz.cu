@@ -290,136 +290,136 @@ oz_outer_kernel(const float2* __restrict__ A, int nk, int nb, long long ld, long
         if (!tc::mbar_wait(&full[i % OZ_NSTAGE], (unsigned)(i / OZ_NSTAGE) & 1u, kOzWaitLimit)) s_fail = 1;
     }
   } else {                               // ---------------- the working warps
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REG_WORK));
-  // this thread's A elements: row r = 8 w + lane % 8, real K 4q .. 4q + 3 with q = lane / 8 and
-  // q + 4, so that a warp's 8-byte slice stores cover 256 contiguous bytes (no bank conflicts)
-  const int r = 8 * w + (lane & 7), q = lane >> 3;
-  const uint32_t lane_col = ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(NACC * (w >> 2));
-  long long acc[NACC];
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REG_WORK));
+    // this thread's A elements: row r = 8 w + lane % 8, real K 4q .. 4q + 3 with q = lane / 8 and
+    // q + 4, so that a warp's 8-byte slice stores cover 256 contiguous bytes (no bank conflicts)
+    const int r = 8 * w + (lane & 7), q = lane >> 3;
+    const uint32_t lane_col = ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(NACC * (w >> 2));
+    long long acc[NACC];
 
-  auto load_a = [&](int c, int kend, long long g, float4 (&v)[2]) {
-    const float2* x = A + (long long)(c * 16 + 2 * q) * ld + g;
+    auto load_a = [&](int c, int kend, long long g, float4 (&v)[2]) {
+      const float2* x = A + (long long)(c * 16 + 2 * q) * ld + g;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int k = c * 16 + 2 * (q + 4 * i);
-      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (g < ng) {
-        if (k < kend) { const float2 y = x[8 * i * ld]; t.x = y.x; t.y = y.y; }
-        if (k + 1 < kend) { const float2 y = x[(8 * i + 1) * ld]; t.z = y.x; t.w = y.y; }
-      }
-      v[i] = t;
-    }
-  };
-  // the SA slices of this thread's 8 values into stage `st`
-  auto store_a = [&](unsigned char* st, const float4 (&v)[2], float sa) {
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      float x[4] = {v[i].x * sa, v[i].y * sa, v[i].z * sa, v[i].w * sa};
-      const int off = oz_off(r, 4 * (q + 4 * i));
-#pragma unroll
-      for (int s = 0; s < O::SA; ++s) {
-        float d[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          d[e] = round_int(x[e]);
-          x[e] = (x[e] - d[e]) * (float)(1 << OZ_BETA);
+      for (int i = 0; i < 2; ++i) {
+        const int k = c * 16 + 2 * (q + 4 * i);
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (g < ng) {
+          if (k < kend) { const float2 y = x[8 * i * ld]; t.x = y.x; t.y = y.y; }
+          if (k + 1 < kend) { const float2 y = x[(8 * i + 1) * ld]; t.z = y.x; t.w = y.y; }
         }
-        const __half2 h01 = __floats2half2_rn(d[0], d[1]), h23 = __floats2half2_rn(d[2], d[3]);   // exact
-        uint2 u;
-        u.x = *reinterpret_cast<const uint32_t*>(&h01);
-        u.y = *reinterpret_cast<const uint32_t*>(&h23);
-        *reinterpret_cast<uint2*>(st + s * O::A_SLICE + off) = u;
+        v[i] = t;
       }
-    }
-  };
-  auto drain = [&]() {
-    tc::fence_after_sync();
+    };
+    // the SA slices of this thread's 8 values into stage `st`
+    auto store_a = [&](unsigned char* st, const float4 (&v)[2], float sa) {
 #pragma unroll
-    for (int wt = 2; wt <= T; ++wt) {
-      const uint32_t ta = tmem + lane_col + (uint32_t)((wt - 2) * O::TN);
-      const int sh = OZ_BETA * (T - wt);
+      for (int i = 0; i < 2; ++i) {
+        float x[4] = {v[i].x * sa, v[i].y * sa, v[i].z * sa, v[i].w * sa};
+        const int off = oz_off(r, 4 * (q + 4 * i));
 #pragma unroll
-      for (int o = 0; o < NACC; o += 8) {                  // eight at a time: the sums hold half of the registers
-        uint32_t v[8];
-        tc::tmem_ld8(ta + (uint32_t)o, v);
-        tc::tmem_wait_ld();
+        for (int s = 0; s < O::SA; ++s) {
+          float d[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[o + j] += (long long)__float2int_rn(__uint_as_float(v[j])) << sh;
+          for (int e = 0; e < 4; ++e) {
+            d[e] = round_int(x[e]);
+            x[e] = (x[e] - d[e]) * (float)(1 << OZ_BETA);
+          }
+          const __half2 h01 = __floats2half2_rn(d[0], d[1]), h23 = __floats2half2_rn(d[2], d[3]);   // exact
+          uint2 u;
+          u.x = *reinterpret_cast<const uint32_t*>(&h01);
+          u.y = *reinterpret_cast<const uint32_t*>(&h23);
+          *reinterpret_cast<uint2*>(st + s * O::A_SLICE + off) = u;
+        }
       }
-    }
-    tc::fence_before_sync();
-  };
+    };
+    auto drain = [&]() {
+      tc::fence_after_sync();
+#pragma unroll
+      for (int wt = 2; wt <= T; ++wt) {
+        const uint32_t ta = tmem + lane_col + (uint32_t)((wt - 2) * O::TN);
+        const int sh = OZ_BETA * (T - wt);
+#pragma unroll
+        for (int o = 0; o < NACC; o += 8) {                  // eight at a time: the sums hold half of the registers
+          uint32_t v[8];
+          tc::tmem_ld8(ta + (uint32_t)o, v);
+          tc::tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[o + j] += (long long)__float2int_rn(__uint_as_float(v[j])) << sh;
+        }
+      }
+      tc::fence_before_sync();
+    };
 
-  auto wait = [&](int n) {               // bounded wait for the MMAs of chunk n of the stream
-    if (!tc::mbar_wait(&bar[n % OZ_NSTAGE], (unsigned)(n / OZ_NSTAGE) & 1u, kOzWaitLimit)) s_fail = 1;
-    return !s_fail;
-  };
-  auto arrive = [&](uint64_t* b) {       // one arrival per warp, after all its lanes
-    __syncwarp();
-    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(b)) : "memory");
-  };
-  auto output = [&](int tile) {          // a finished tile, then zero sums
-    const int row = 32 * (w & 3) + lane, b0 = (tile % nbt) * O::BB;
-    const long long gg = (long long)(tile / nbt) * OZ_TM + row;
-    const int ri = (w >> 2) >= 2 ? 1 : 0;                 // column groups 0-1 real, 2-3 imaginary
-    const int jq = ((w >> 2) & 1) * NACC;
-    if (gg < ng) {
-      const int ergg = erow[gg];
+    auto wait = [&](int n) {               // bounded wait for the MMAs of chunk n of the stream
+      if (!tc::mbar_wait(&bar[n % OZ_NSTAGE], (unsigned)(n / OZ_NSTAGE) & 1u, kOzWaitLimit)) s_fail = 1;
+      return !s_fail;
+    };
+    auto arrive = [&](uint64_t* b) {       // one arrival per warp, after all its lanes
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(b)) : "memory");
+    };
+    auto output = [&](int tile) {          // a finished tile, then zero sums
+      const int row = 32 * (w & 3) + lane, b0 = (tile % nbt) * O::BB;
+      const long long gg = (long long)(tile / nbt) * OZ_TM + row;
+      const int ri = (w >> 2) >= 2 ? 1 : 0;                 // column groups 0-1 real, 2-3 imaginary
+      const int jq = ((w >> 2) & 1) * NACC;
+      if (gg < ng) {
+        const int ergg = erow[gg];
 #pragma unroll
-      for (int j = 0; j < NACC; ++j) {
-        const int b = b0 + jq + j;
-        if (b < nb) {
-          const int e = ergg + fcol[b] - OZ_BETA * T;
-          if constexpr (sizeof(OUT) == 8)   // one rounding of the exact integer, then an exact power of two
-            reinterpret_cast<float*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexpf(__ll2float_rn(acc[j]), e);
-          else
-            reinterpret_cast<double*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexp(__ll2double_rn(acc[j]), e);
+        for (int j = 0; j < NACC; ++j) {
+          const int b = b0 + jq + j;
+          if (b < nb) {
+            const int e = ergg + fcol[b] - OZ_BETA * T;
+            if constexpr (sizeof(OUT) == 8)   // one rounding of the exact integer, then an exact power of two
+              reinterpret_cast<float*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexpf(__ll2float_rn(acc[j]), e);
+            else
+              reinterpret_cast<double*>(Out)[2 * ((long long)b * ld + gg) + ri] = ldexp(__ll2double_rn(acc[j]), e);
+          }
+          if (j % 4 == 3) asm volatile("" ::: "memory");     // a few loads at a time: registers are short
         }
-        if (j % 4 == 3) asm volatile("" ::: "memory");     // a few loads at a time: registers are short
       }
-    }
+#pragma unroll
+      for (int j = 0; j < NACC; ++j) acc[j] = 0;
+    };
+    float4 cur[2];
+    int n = 0, due = -1;                   // chunk of the stream; tile that ends with the pending group
+    bool pending = false, ok = true;       // a group ended with chunk n - 1
 #pragma unroll
     for (int j = 0; j < NACC; ++j) acc[j] = 0;
-  };
-  float4 cur[2];
-  int n = 0, due = -1;                   // chunk of the stream; tile that ends with the pending group
-  bool pending = false, ok = true;       // a group ended with chunk n - 1
-#pragma unroll
-  for (int j = 0; j < NACC; ++j) acc[j] = 0;
-  int next_e = 0;                        // exponent of this thread's row in the next tile
-  if ((int)blockIdx.x < ntiles) {
-    const long long g = (long long)(blockIdx.x / nbt) * OZ_TM + r;
-    load_a(0, kend_of(blockIdx.x), g, cur);
-    next_e = g < ng ? erow[g] : 0;
-  }
-  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-    const int kend = kend_of(tile), nchunks = (kend + 15) / 16, next = tile + gridDim.x;
-    const long long g = (long long)(tile / nbt) * OZ_TM + r, gn = (long long)(next / nbt) * OZ_TM + r;
-    const float sa = ldexpf(1.0f, OZ_BETA - next_e);       // exact power of two
-    if (next < ntiles) next_e = gn < ng ? erow[gn] : 0;
-    for (int c = 0; c < nchunks; ++c, ++n) {
-      const bool last = c == nchunks - 1;
-      if (n >= OZ_NSTAGE && !wait(n - OZ_NSTAGE)) { ok = false; break; }
-      store_a(base + (n % OZ_NSTAGE) * O::STAGE, cur, sa);
-      tc::fence_async_smem();
-      arrive(&ready[n % OZ_NSTAGE]);
-      if (!last) load_a(c + 1, kend, g, cur);
-      else if (next < ntiles) load_a(0, kend_of(next), gn, cur);
-      if (pending) {
-        if (!wait(n - 1)) { ok = false; break; }
-        drain();
-        arrive(drained);
-        if (due >= 0) output(due);
+    int next_e = 0;                        // exponent of this thread's row in the next tile
+    if ((int)blockIdx.x < ntiles) {
+      const long long g = (long long)(blockIdx.x / nbt) * OZ_TM + r;
+      load_a(0, kend_of(blockIdx.x), g, cur);
+      next_e = g < ng ? erow[g] : 0;
+    }
+    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+      const int kend = kend_of(tile), nchunks = (kend + 15) / 16, next = tile + gridDim.x;
+      const long long g = (long long)(tile / nbt) * OZ_TM + r, gn = (long long)(next / nbt) * OZ_TM + r;
+      const float sa = ldexpf(1.0f, OZ_BETA - next_e);       // exact power of two
+      if (next < ntiles) next_e = gn < ng ? erow[gn] : 0;
+      for (int c = 0; c < nchunks; ++c, ++n) {
+        const bool last = c == nchunks - 1;
+        if (n >= OZ_NSTAGE && !wait(n - OZ_NSTAGE)) { ok = false; break; }
+        store_a(base + (n % OZ_NSTAGE) * O::STAGE, cur, sa);
+        tc::fence_async_smem();
+        arrive(&ready[n % OZ_NSTAGE]);
+        if (!last) load_a(c + 1, kend, g, cur);
+        else if (next < ntiles) load_a(0, kend_of(next), gn, cur);
+        if (pending) {
+          if (!wait(n - 1)) { ok = false; break; }
+          drain();
+          arrive(drained);
+          if (due >= 0) output(due);
+        }
+        pending = last || c % OZ_GROUP == OZ_GROUP - 1;
+        due = last ? tile : -1;
       }
-      pending = last || c % OZ_GROUP == OZ_GROUP - 1;
-      due = last ? tile : -1;
+    }
+    if (ok && pending && wait(n - 1)) {
+      drain();
+      output(due);
     }
   }
-  if (ok && pending && wait(n - 1)) {
-    drain();
-    output(due);
-  }
-  }   // working warps
   __syncthreads();
   if (s_fail && tid == 0) {
     status[0] = -6;   // ACE_ERR_TIMEOUT
