@@ -883,7 +883,10 @@ EncodeFn encoder() {
   static const EncodeFn f = [] {
     void* e = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &e, 12000, cudaEnableDefault, &q) != cudaSuccess) e = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &e, 12000, cudaEnableDefault, &q) != cudaSuccess) {
+      cudaGetLastError();   // no error of the plan's: the TF32 products serve
+      e = nullptr;
+    }
     return reinterpret_cast<EncodeFn>(e);
   }();
   return f;
