@@ -250,7 +250,7 @@ ace_status ace_poisson(ace_plan* plan, const void* rho, int n_b, void* V, void* 
  * captured CUDA graph. The systems are spread over `chains` concurrent
  * streams (0 = 3), longest first, each to the chain with the least estimated
  * work (N(N+1)/2 N_g); inside a chain they run in turn, each with its own
- * two-stream pair schedule. The graph is cached process-wide under all the
+ * pair schedule. The graph is cached process-wide under all the
  * pointers (plans, Phi[i], Xi[i], Ex, ws) and replayed on later calls.
  * plans: n_sys distinct plans on the current device. Phi[i], Xi[i]: N_i
  * vectors of plan i's layout (device, 16-byte aligned). Ex: NULL or device
@@ -265,8 +265,8 @@ ace_status ace_build_batched(ace_plan* const* plans, const void* const* Phi, voi
 /* Autotuner (schedule choice only; results are the same for every choice up
  * to FP32 rounding order): times ace_build of the descriptor's problem on the
  * current device for each candidate schedule -- tile edge 8, 6 or 4 orbitals,
- * pair-batch scratch of about 36, 72 or 144 MiB, the two-stream overlapped
- * pair schedule or two lanes without overlap, and (C64 plans) the radix order
+ * pair-batch scratch of about 36, 72 or 144 MiB, the overlapped pair schedule
+ * (ACE_FLAG_NO_OVERLAP says which form that is) or two lanes without overlap, and (C64 plans) the radix order
  * of the line transforms (ACE_FLAG_RADIX_ODD_FIRST) -- on seeded pseudo-random
  * orbitals, `reps` timed builds each (0 = 3) after one untimed build, and
  * writes the fastest into *best (a copy of *d with tile, max_pairs, lanes and

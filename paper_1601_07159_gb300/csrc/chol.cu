@@ -22,8 +22,8 @@
 // cycles per warp instruction and SM quadrant), and at 128 orbitals and fewer its latency: outputs are
 // spread over as many SMs as there are (2-row panels and 8 x 8 tiles in place of 16 rows
 // and 16 x 16), sums are cut in parts that meet by shuffles, and dependent steps
-// are few. Kernel times for 128 orbitals: 392 -> 212 us (diag 8 x 22.4 -> 10.7, panel 8.1 ->
-// 5.0, update 8.2 -> 5.3, the inverse from 7 row steps of 12.9 to 3 levels of 15.7).
+// are few. Kernel times for 128 orbitals: 392 -> 239 us (diag 8 x 22.4 -> 14.2, panel 8.1 ->
+// 4.9, update 8.2 -> 5.2, the inverse from 7 row steps of 12.9 to 3 levels of 16.0).
 // Every kernel returns at once when the status word already holds a failure.
 #include <cmath>
 
@@ -82,7 +82,7 @@ __device__ __forceinline__ double minus_abs2(double a, double2 u, double r) {
 // the step before (two buffers, one barrier a step). Warp PIV works ahead on the
 // pivot: d_{j+1} = a_{j+1,j+1} - |a_{j+1,j}|^2 / d_j and its reciprocal, while the
 // others do step j (with the pivot taken from its element's thread and the inverse
-// formed afterwards, by recursive doubling, the kernel took 22.4 us; 10.7 so). What it
+// formed afterwards, by recursive doubling, the kernel took 22.4 us; 14.2 so). What it
 // leaves for a step (the pivot's reciprocal and verdict) lies in the word of that
 // step's parity, which no thread reads before the barrier.
 // At the end L_ik = a_ik / sqrt(d_k), and row i of X is divided by sqrt(d_i). Reciprocals
