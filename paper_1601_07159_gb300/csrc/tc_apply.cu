@@ -8,9 +8,10 @@
 // 2018, with both parts scaled). hi and lo carry 22 to 23 bits of every value down to
 // 2^-18 of the row's largest (lo is then a normal FP16 number) and below that an absolute
 // error of 2^-40 of the largest. So what shares a scale matters: the gram product's
-// rows and columns are vectors, scaled anew every 512 points; the outer product's rows are points (the largest value
-// of any orbital there), so that V_ACE psi keeps its relative accuracy where every
-// orbital is small, as in vacuum, and its columns are the bands' coefficients.
+// rows and columns are vectors, scaled anew every 512 points; the outer product's rows
+// are points (the largest value of any orbital there), so that V_ACE psi keeps its
+// relative accuracy where every orbital is small, as in vacuum, and its columns are the
+// bands' coefficients.
 // Three products hi hi + hi lo + lo hi are kept; the dropped lo lo is below
 // 2^-24. (The TF32 split of tc_gemm.cu truncates both parts and drops 2^-20.) A
 // kind::f16 MMA does twice the work of a kind::tf32 one per cycle on half the
@@ -205,9 +206,12 @@ template <int TN> struct Stream {
     for (int i = 0; i < Tile<TN>::NH; ++i) re[i] = im[i] = 0.f;
   }
   // bounded wait for the MMAs of stage s, then the sums of a finished group, whose units
-  // `units` gives the sums so far
-  template <typename F> __device__ __forceinline__ bool settle(int s, F&& units) {
-    if (!tc::mbar_wait(&bar[s], (phase >> s) & 1u, kWaitLimit)) return false;
+  // `units` gives the sums so far. VOTE: `units` exchanges values within the warp, so
+  // that a lost wait has to take all its lanes along.
+  template <bool VOTE, typename F> __device__ __forceinline__ bool settle(int s, F&& units) {
+    bool done = tc::mbar_wait(&bar[s], (phase >> s) & 1u, kWaitLimit);
+    if (VOTE) done = __all_sync(0xffffffffu, done);
+    if (!done) return false;
     phase ^= 1u << s;
     issued &= ~(1u << s);
     const unsigned d = (drain >> (2 * s)) & 3u;
@@ -247,10 +251,10 @@ template <int TN> __device__ __forceinline__ void teardown(uint32_t tmem) {
 // Largest |component| (as float bits, which order like the values; NaN is skipped) of
 // each vector, mx[0 .. na) for A and mx[na ..) for B, and of each point over the vectors
 // of A, pt[g]; the biased exponent of each vector's largest in each segment, sx[segment *
-// row + vector], with the vectors of B from `at_b` on. Grid: (ya parts of `per` vectors of A and then those of B, 512-point
-// segments). A warp takes a segment of one vector at a time, eight 16-byte loads in flight a
-// thread, and keeps the maxima of its points in registers; one sweep of the vectors,
-// bound by memory.
+// row + vector], with the vectors of B from `at_b` on. Grid: (ya parts of `per` vectors
+// of A and then those of B, 512-point segments). A warp takes a segment of one vector at
+// a time, eight 16-byte loads in flight a thread, and keeps the maxima of its points in
+// registers; one sweep of the vectors, bound by memory.
 constexpr int SEG = 512, kMaxPart = 64;
 __global__ void __launch_bounds__(256)
 maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B, int nb, long long ld, long long ng,
@@ -319,8 +323,8 @@ maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B
 // the vectors' largest values keep their accuracy: accumulator groups end where
 // segments do, and when a segment's boosts differ from those of the sums so far, the
 // sums are taken to its units first (a multiplication by a power of two). The split's
-// sums are left in the units of the vectors. A segment's
-// exponents arrive with its first chunk.
+// sums are left in the units of the vectors. A segment's exponents arrive with its
+// first chunk. Costs 4 of 96 us at 48^3, 128 x 192, 0.7 of 36 at 16 x 24.
 template <int TN>
 __global__ void __launch_bounds__(Tile<TN>::G_THREADS, 1)
 gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_constant__ CUtensorMap B, int nb, long long ng,
@@ -455,7 +459,7 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
         split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g0), sb, bh[0], bl[0]);
         split4(*reinterpret_cast<const float4*>(raw + TM * KC * 4 + g1), sb, bh[1], bl[1]);
       }
-      if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;   // the MMAs of chunk c - ST read this stage
+      if (((S.issued >> s) & 1u) && !S.template settle<true>(s, units)) s_fail = 1;   // the MMAs of chunk c - ST read this stage
 #pragma unroll
       for (int i = 0; i < 2; ++i) {                        // granule i: K values 4 q + 16 i ..
         *reinterpret_cast<uint2*>(st + i * 256) = ah[i];
@@ -477,7 +481,7 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
         __syncwarp();
         if (lane == 0)
           asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar + ST + R + s)) : "memory");
-        if (s_fail) {
+        if (__any_sync(0xffffffffu, s_fail)) {           // the warp leaves as one
           ok = false;
           break;
         }
@@ -499,7 +503,7 @@ gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_consta
     }
     for (int i = 0; i < ST; ++i) {                         // the last commits, in chunk order
       const int s = (nchunks + i) % ST;
-      if (((S.issued >> s) & 1u) && !S.settle(s, units)) s_fail = 1;
+      if (((S.issued >> s) & 1u) && !S.template settle<true>(s, units)) s_fail = 1;
     }
     if (!IW && !ok)                                        // copies in flight (bounded)
       for (int i = 0; i < R; ++i) tc::mbar_wait(bar + ST + i, (lphase >> i) & 1u, 1u << 16);
@@ -703,7 +707,7 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nb, long long ld, long
   int due0 = -1, due1 = -1;                              // tile that ends with the pending commit of stage 0, 1
   unsigned lphase = 0;                                   // parities of the landing barriers
   auto finish = [&](int s) {                             // the pending commit of stage s, and the stores that it ends
-    if (!S.settle(s, [] {})) {
+    if (!S.template settle<false>(s, [] {})) {
       s_fail = 1;
       return;
     }
@@ -773,7 +777,7 @@ outer16_kernel(const __grid_constant__ CUtensorMap A, int nb, long long ld, long
     }
   } else {
     for (int s = 0; s < 2; ++s)
-      if ((S.issued >> s) & 1u) S.settle(s, [] {});
+      if ((S.issued >> s) & 1u) S.template settle<false>(s, [] {});
     for (int i = 0; i < R; ++i)                          // copies in flight (bounded)
       tc::mbar_wait(bar + 2 + i, (lphase >> i) & 1u, 1u << 16);
   }
