@@ -209,12 +209,12 @@ template <int TN> struct Stream {
   // `units` gives the sums so far. VOTE: `units` exchanges values within the warp, so
   // that a lost wait has to take all its lanes along.
   template <bool VOTE, typename F> __device__ __forceinline__ bool settle(int s, F&& units) {
+    const unsigned d = (drain >> (2 * s)) & 3u;
     bool done = tc::mbar_wait(&bar[s], (phase >> s) & 1u, kWaitLimit);
-    if (VOTE) done = __all_sync(0xffffffffu, done);
+    if (VOTE && d) done = __all_sync(0xffffffffu, done);
     if (!done) return false;
     phase ^= 1u << s;
     issued &= ~(1u << s);
-    const unsigned d = (drain >> (2 * s)) & 3u;
     if (d) {
       units();
       tc::fence_after_sync();
