@@ -37,9 +37,9 @@
 // are added in FP32 registers while the next group's MMAs run. Every mbarrier wait
 // is bounded, as in tc_gemm.cu.
 //
-// Measured, TF32 split -> this: 48^3, 128 orbitals, 192 bands: gram 169 -> 96 us, outer
-// 188 -> 100 us, the sweep over the vectors for their maxima 43 us (6.5 TB/s), whole
-// call 378 -> 278 us; 96^3, 1024 x 1536: 116 -> 71.4 ms (gram 37.5, outer 31.3, maxima 2.4).
+// Measured, TF32 split -> this: 48^3, 128 orbitals, 192 bands: gram 169 -> 98 us, outer
+// 188 -> 101 us, the sweep over the vectors for their maxima 44 us (6.5 TB/s), whole
+// call 378 -> 281 us; 96^3, 1024 x 1536: 116 -> 68.7 ms (gram 37.5, outer 28.4, maxima 2.4).
 // With the MMAs and the conversion switched off the 48^3 loops take 67 us (gram) and 95
 // (outer, with a scale per value) (387 and 553 MB through L2, 5.8 TB/s): tile traffic
 // bounds them, then the chain convert - fence - barrier - issue of a chunk. Relative error
@@ -79,7 +79,8 @@ template <int TN> struct Tile {
   static constexpr int G_RAW = (TM + BB) * KC * 4;
   // The narrow tiles' chunks are short beside a block-wide barrier and the issue of their
   // MMAs: a warp of its own fetches and issues, and the working warps meet it on
-  // mbarriers (16 x 24 vectors of 48^3: 38.0 us without, 35.6 us with). The wide ones need
+  // mbarriers (16 x 24 vectors of 48^3, with one scale per vector: 38.0 us without, 35.6 us
+  // with; 36.1 with the segments' scales). The wide ones need
   // the registers that a fifth warp per SM quadrant takes.
   static constexpr bool G_ISSUER = TN <= 128;
   static constexpr int G_THREADS = THREADS + (G_ISSUER ? 128 : 0);
@@ -324,7 +325,7 @@ maxima_kernel(const float2* __restrict__ A, int na, const float2* __restrict__ B
 // segments do, and when a segment's boosts differ from those of the sums so far, the
 // sums are taken to its units first (a multiplication by a power of two). The split's
 // sums are left in the units of the vectors. A segment's exponents arrive with its
-// first chunk. Costs 4 of 96 us at 48^3, 128 x 192, 0.7 of 36 at 16 x 24.
+// first chunk. Costs 5 of 98 us at 48^3, 128 x 192, 0.8 of 36 at 16 x 24.
 template <int TN>
 __global__ void __launch_bounds__(Tile<TN>::G_THREADS, 1)
 gram16_kernel(const __grid_constant__ CUtensorMap A, int na, const __grid_constant__ CUtensorMap B, int nb, long long ng,
